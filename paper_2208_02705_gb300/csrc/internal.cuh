@@ -188,7 +188,7 @@ struct MlpWeights {
     const float *w32;          // FP32 masters [F][P]
     const float *wt;           // FP32 transposed/padded copy for SIMT [F][Pt]
     int64_t Pt;
-    const float *wr;           // FP32 row-padded copy ([out][round4(in)]) for the SIMT adjoint [F][Pr]
+    const float *wr;           // FP32 copy ([out][W inputs] per layer) for the SIMT adjoint's dgrad [F][Pr]
     int64_t Pr;
     const void *wimg;          // BF16 tensor-core images [F][img_bytes]
     int64_t img_bytes;
@@ -257,6 +257,7 @@ void launch_composite_bwd(int64_t n_rays, int R, const uint32_t *cnt, const uint
 void launch_mlp_bwd_simt(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr,
                          const float4 *gsr, float *grad, int grid, cudaStream_t s);
 bool mlp_bwd_supported(int W, int H);
+int mlp_bwd_simt_tile(int W, int H);      // samples per tile of the SIMT adjoint's bucketing
 // tcgen05 BF16 adjoint (W <= 64 and the shared-memory budget: W = 32 with
 // H <= 4, W = 64 with H <= 3); needs the BF16 weight images
 bool mlp_bwd_tc_supported(int W, int H);

@@ -1,138 +1,124 @@
-// Adjoint of the per-field tiny MLPs for the fine-tuning step (Sec.
+// FP32 adjoint of the per-field tiny MLPs for the fine-tuning step (Sec.
 // "Adaptive Radiance Fields Slimming and Fine-tuning": L2 loss on rendered
-// pixels), FP32 SIMT: one thread per sample, tiles of 128 samples of one
-// field.  Each thread recomputes its sample's encoding and activations (they
-// are never stored between passes), then walks the layers backwards:
-//   dgrad  dx = W^T dz            (per thread, weights from a row-padded copy)
-//   wgrad  dW += dz^T x, db += dz (per tile: the 128 rows of x and dz are
-//                                  staged in shared memory and each thread
-//                                  owns a set of (out, in) entries)
-// The field's gradient accumulates in shared memory while the CTA walks its
-// contiguous run of tiles and is added to the global FP32 gradient (one
-// atomic per parameter) whenever the field changes.  Also: the Adam update.
+// pixels) and the distillation step (Eq. 7), as register-tiled SIMT products;
+// the Adam update and the losses.
+//
+// A CTA walks a contiguous run of tiles of kS samples of one field.  Per tile
+// it recomputes the encoding and every activation (nothing is stored between
+// the passes), then walks the layers backwards:
+//   dgrad  dX[k][s]  = sum_n W[n][k] dZ[n][s]
+//   wgrad  dW[n][k] += sum_s dZ[n][s] X[k][s],  db[n] += sum_s dZ[n][s]
+// What bounds it: the FP32 FMA pipe (2 x (3 MACs - 63 W) FLOP per sample,
+// 126 kFLOP at W = 64 / H = 3).  So
+//  - every activation of the tile stays in shared memory, feature-major
+//    ([k][kS samples], rows kS + 4 apart: consecutive rows start 4 banks
+//    apart, which keeps the wgrad's loads along s conflict-free); dZ of a
+//    layer overwrites the activations it belongs to, so no second buffer;
+//  - a thread owns 4 samples x TN outputs (forward, all 8 warps) or
+//    4 samples x 2 TN (dgrad, warps 0-3), while warps 4-7 form the same
+//    layer's wgrad (W/8 outputs x up to 6 inputs per thread, reduced over s
+//    in pairs): both have about the same work and share the FMA pipe;
+//  - the weights stream through a ring of shared-memory stages (16 rows each),
+//    copied asynchronously by warps 0-3 a few stages ahead, one barrier per
+//    stage: they are read once per tile and would not fit beside the gradient
+//    (bulk copies issued by one thread took ~400 cycles each out of its
+//    warp's products; a producer warp would cap the others at 168 registers);
+//  - the field's gradient accumulates in shared memory and goes to global
+//    memory (one atomic per parameter) when the field changes.
+// kS is what shared memory holds: 64 samples at W = 64 (H <= 3), 32 at
+// W = 64 / H = 4, 128 at W = 32.
 #include "internal.cuh"
 
 namespace roam {
 
 namespace {
 
-constexpr int kThreads = 128;
-
 __host__ __device__ constexpr int round4(int x) { return (x + 3) & ~3; }
 
 // offsets of the API layout
 struct ALayout {
     int64_t l1, hid, head, col, out, total;
-    __host__ __device__ ALayout(int W, int H)
+    __host__ __device__ constexpr ALayout(int W, int H)
+        : l1(0), hid((int64_t)W * kPeX + W), head(hid + (int64_t)(H - 1) * ((int64_t)W * W + W)),
+          col(head + (int64_t)(1 + W) * W + (1 + W)), out(col + (int64_t)W * (W + kPeD) + W),
+          total(out + 3 * (int64_t)W + 3)
     {
-        int64_t o = 0;
-        l1 = o;   o += (int64_t)W * kPeX + W;
-        hid = o;  o += (int64_t)(H - 1) * ((int64_t)W * W + W);
-        head = o; o += (int64_t)(1 + W) * W + (1 + W);
-        col = o;  o += (int64_t)W * (W + kPeD) + W;
-        out = o;  o += 3 * (int64_t)W + 3;
-        total = o;
     }
 };
 
-// offsets of the row-padded copy [out][round4(in)] (matrices only)
+// offsets of the dgrad copy: rows [out][W inputs] of the hidden layers, the
+// head's features (the density row is read from the masters) and the colour
+// layer (its F(d) inputs need no gradient)
 struct RLayout {
-    int64_t l1, hid, head, col, out, total;
-    __host__ __device__ RLayout(int W, int H)
+    int64_t hid, head, col, total;
+    __host__ __device__ constexpr RLayout(int W, int H)
+        : hid(0), head((int64_t)(H - 1) * W * W), col(head + (int64_t)W * W), total(col + (int64_t)W * W)
     {
-        int64_t o = 0;
-        l1 = o;   o += (int64_t)W * round4(kPeX);
-        hid = o;  o += (int64_t)(H - 1) * W * W;
-        head = o; o += (int64_t)(1 + W) * W;
-        col = o;  o += (int64_t)W * round4(W + kPeD);
-        out = o;  o += 3 * (int64_t)W;
-        total = o;
     }
 };
 
 // offsets of the transposed copy used by the forward kernel (same as mlp_simt.cu;
 // the head's row: W features, then the density logit, then zeros)
 struct TLayout {
-    int64_t l1, hid, head, col, out, total;
-    __host__ __device__ TLayout(int W, int H)
+    int64_t l1, hid, head, col;
+    __host__ __device__ constexpr TLayout(int W, int H)
+        : l1(0), hid((int64_t)kPeX * W + W), head(hid + (int64_t)(H - 1) * ((int64_t)W * W + W)),
+          col(head + (int64_t)W * round4(1 + W) + round4(1 + W))
     {
-        int64_t o = 0;
-        l1 = o;   o += (int64_t)kPeX * W + W;
-        hid = o;  o += (int64_t)(H - 1) * ((int64_t)W * W + W);
-        head = o; o += (int64_t)W * round4(1 + W) + round4(1 + W);
-        col = o;  o += (int64_t)(W + kPeD) * W + W;
-        out = o;  o += (int64_t)W * 4 + 4;
-        total = o;
     }
 };
 
-// acc[o] = b[o] + sum_i x[i] WT[i][o], x a per-thread array
-template <int K, int N>
-__device__ __forceinline__ void dense_arr(const float *x, const float *__restrict__ wt, float (&acc)[N])
-{
-    const float4 *b4 = reinterpret_cast<const float4 *>(wt + (int64_t)K * N);
-#pragma unroll
-    for (int q = 0; q < N / 4; ++q) {
-        const float4 bb = __ldg(b4 + q);
-        acc[4 * q + 0] = bb.x; acc[4 * q + 1] = bb.y; acc[4 * q + 2] = bb.z; acc[4 * q + 3] = bb.w;
-    }
-#pragma unroll 1
-    for (int i = 0; i < K; ++i) {
-        const float xi = x[i];
-        const float4 *wr = reinterpret_cast<const float4 *>(wt + (int64_t)i * N);
-#pragma unroll
-        for (int q = 0; q < N / 4; ++q) {
-            const float4 ww = __ldg(wr + q);
-            acc[4 * q + 0] = fmaf(ww.x, xi, acc[4 * q + 0]);
-            acc[4 * q + 1] = fmaf(ww.y, xi, acc[4 * q + 1]);
-            acc[4 * q + 2] = fmaf(ww.z, xi, acc[4 * q + 2]);
-            acc[4 * q + 3] = fmaf(ww.w, xi, acc[4 * q + 3]);
-        }
-    }
-}
+template <int V>
+struct Int {
+    static constexpr int value = V;
+};
 
-// dx[k] = sum_n W[n][k] dz[n]; W row-padded [N][KP]; dz in the thread's
-// shared-memory row
-template <int N, int KP>
-__device__ __forceinline__ void dgrad(const float *dz_row, const float *__restrict__ wr, float (&dx)[KP])
-{
-#pragma unroll
-    for (int k = 0; k < KP; ++k) dx[k] = 0.f;
-#pragma unroll 1
-    for (int n = 0; n < N; ++n) {
-        const float dn = dz_row[n];
-        const float4 *w4 = reinterpret_cast<const float4 *>(wr + (int64_t)n * KP);
-#pragma unroll
-        for (int q = 0; q < KP / 4; ++q) {
-            const float4 ww = __ldg(w4 + q);
-            dx[4 * q + 0] = fmaf(ww.x, dn, dx[4 * q + 0]);
-            dx[4 * q + 1] = fmaf(ww.y, dn, dx[4 * q + 1]);
-            dx[4 * q + 2] = fmaf(ww.z, dn, dx[4 * q + 2]);
-            dx[4 * q + 3] = fmaf(ww.w, dn, dx[4 * q + 3]);
-        }
-    }
-}
+constexpr int kThreads = 256;
+constexpr int kRingRows = 16;       // weight rows per ring stage
 
-// dW[n][k] += sum_s dz[s][n] x[s][k], db[n] += sum_s dz[s][n], over the
-// tile's staged rows; each entry is owned by one thread
-template <int N, int K, int XS, int DS>
-__device__ __forceinline__ void wgrad(const float *xs, const float *dzs, float *gw, float *gb, int tid)
-{
-    for (int e = tid; e < N * K + N; e += kThreads) {
-        float acc = 0.f;
-        if (e < N * K) {
-            const int n = e / K, k = e - n * K;
-#pragma unroll 8
-            for (int s = 0; s < kThreads; ++s) acc = fmaf(dzs[s * DS + n], xs[s * XS + k], acc);
-            gw[e] += acc;
-        } else {
-            const int n = e - N * K;
-#pragma unroll 8
-            for (int s = 0; s < kThreads; ++s) acc += dzs[s * DS + n];
-            gb[n] += acc;
-        }
-    }
-}
+template <int W, int H>
+struct FbShape {
+    static constexpr int S = W == 32 ? 128 : (H <= 3 ? 64 : 32);    // samples per tile
+    static constexpr int XS = S + 4;                                  // row stride of the activations
+    static constexpr int TN = W * S / 1024;                           // forward outputs per thread
+    static constexpr int TD = 2 * TN;                                 // dgrad inputs per thread
+    static constexpr int KC = W + kPeD;
+    static constexpr int NH = round4(1 + W);
+    // activation rows: F(x), h_1 .. h_H, [feat; F(d)], g
+    static constexpr int rX = 0;
+    __host__ __device__ static constexpr int rH(int j) { return kPeX + (j - 1) * W; }    // h_j, j >= 1
+    static constexpr int rC = kPeX + H * W;
+    static constexpr int rG = rC + KC;
+    static constexpr int kRows = rG + W;
+    // gradient accumulators: rows of each matrix 4 or -4 banks apart
+    static constexpr int SA = 68, SH = W + 4, SC = W == 64 ? 92 : 60;
+    static constexpr int gA = 0;
+    static constexpr int gHid = gA + W * SA;
+    static constexpr int gHead = gHid + (H - 1) * W * SH;    // W feature rows
+    static constexpr int gCol = gHead + W * SH;
+    static constexpr int gDen = gCol + W * SC;               // the head's density row, W
+    static constexpr int gOut = gDen + W;                    // 3 x W
+    static constexpr int gB = gOut + 3 * W;                  // biases: (H + 2) x W (L1, hidden, head features, colour)
+    static constexpr int gBd = gB + (H + 2) * W;             // density bias, then 3 output biases
+    static constexpr int kGrad = round4(gBd + 4);
+    // the field's small tables: biases as above, density weights, output
+    // weights, density bias and output biases
+    static constexpr int tB = 0;
+    static constexpr int tDen = tB + (H + 2) * W;
+    static constexpr int tOut = tDen + W;
+    static constexpr int tBd = tOut + 3 * W;
+    static constexpr int kTab = round4(tBd + 4);
+    static constexpr int kStage = kRingRows * NH;            // floats of one ring stage
+    static constexpr int kFixed = kRows * XS + kGrad + kTab + 4 * S;     // + dz of the 3 outputs and the density
+    static constexpr int kStages = ((227 * 1024 - 1024) / 4 - kFixed) / kStage < 6
+                                       ? ((227 * 1024 - 1024) / 4 - kFixed) / kStage : 6;
+    static constexpr size_t kSmem = (size_t)(kFixed + kStages * kStage) * sizeof(float);
+    // ring stages per tile: forward rows of every layer, then the dgrad's
+    static constexpr int kPer = (kPeX + kRingRows - 1) / kRingRows + H * (W / kRingRows) +
+                                (KC + kRingRows - 1) / kRingRows + (H + 1) * (W / kRingRows);
+    static_assert(kStages >= 4, "the weight ring keeps a few stages in flight");
+    static_assert(TN == 2 || TN == 4, "forward tiles of 2 or 4 outputs");
+};
 
 __device__ __forceinline__ float local_coord(float th0, float delta, float o, float dh, float dl, float scale,
                                              float offset)
@@ -150,265 +136,529 @@ __device__ __forceinline__ float local_coord(float th0, float delta, float o, fl
     return __fadd_rn(__fadd_rn(qh, offset), ql);
 }
 
-template <int L>
-__device__ __forceinline__ void encode_arr(float x0, float x1, float x2, float *e)
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
 {
-    e[0] = x0; e[1] = x1; e[2] = x2;
-    const float xs[3] = {x0, x1, x2};
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+// TN consecutive floats from shared memory
+template <int TN>
+__device__ __forceinline__ void ld_row(const float *p, float2 (&w)[TN / 2])
+{
+    if constexpr (TN >= 4) {
 #pragma unroll
-    for (int k = 0; k < L; ++k) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            float s, c;
-            sincospif(ldexpf(xs[a], k), &s, &c);
-            e[3 + 6 * k + a] = s;
-            e[6 + 6 * k + a] = c;
+        for (int q = 0; q < TN / 4; ++q) {
+            const float4 v = *reinterpret_cast<const float4 *>(p + 4 * q);
+            w[2 * q] = make_float2(v.x, v.y);
+            w[2 * q + 1] = make_float2(v.z, v.w);
         }
+    } else {
+        w[0] = *reinterpret_cast<const float2 *>(p);
     }
 }
 
-template <int N>
-__device__ __forceinline__ void stage_row(float *row, const float (&v)[N], int n)
+// One tile's sample of this thread (thread t of a group of kS takes sample
+// t mod kS), gathered in stages a tile ahead so that no stage waits for the
+// load before it.
+struct FbPending {
+    bool on;
+    uint32_t idx, rec, ray;
+    float4 o, d, dl;
+};
+
+__device__ __forceinline__ void fb_index(FbPending &q, const BucketBufs &b, const Tile &tl, int s, bool more)
 {
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-        if (i < n) row[i] = v[i];
+    q.on = more && (uint32_t)s < tl.count;
+    if (q.on) q.idx = b.sorted[tl.start + s];
+}
+
+__device__ __forceinline__ void fb_record(FbPending &q, const SampleSrc &src)
+{
+    if (!q.on || src.mode != 0) return;
+    const uint32_t i = group_of(q.idx >> 5, (uint32_t)src.R) * 32u + (q.idx & 31u);
+    q.rec = src.recs[q.idx];
+    q.ray = src.live ? src.live[i] : i;
+}
+
+__device__ __forceinline__ void fb_ray(FbPending &q, const SampleSrc &src)
+{
+    if (!q.on) return;
+    if (src.mode == 0) {
+        q.o = src.st.orig[q.ray];
+        q.d = src.st.dir[q.ray];
+        if (src.accurate) q.dl = src.st.dir_lo[q.ray];
+    } else {
+        const int64_t k = 3 * (int64_t)q.idx;
+        q.o = make_float4(src.p[k], src.p[k + 1], src.p[k + 2], 0.f);
+        q.d = make_float4(src.d[k], src.d[k + 1], src.d[k + 2], 0.f);
+    }
 }
 
 template <int W, int H>
-__global__ void __launch_bounds__(kThreads, 1) k_mlp_bwd_simt(MlpWeights w, SampleSrc src, BucketBufs b,
-                                                              Counters *ctr, const float4 *gsr, float *grad)
+__global__ void __launch_bounds__(kThreads, 1)
+    k_mlp_bwd_simt(MlpWeights w, SampleSrc src, BucketBufs b, Counters *ctr, const float4 *gsr, float *grad)
 {
-    constexpr int KC = W + kPeD;
-    constexpr int KMAX = KC > kPeX ? KC : kPeX;
-    constexpr int XS = KMAX + 1;
-    constexpr int DS = W + 2;
-    constexpr int NH = round4(1 + W);
-    const ALayout A(W, H);
-    const RLayout RL(W, H);
-    const TLayout TL(W, H);
-    const int P = (int)A.total;
-    extern __shared__ float smem[];
-    float *gacc = smem;                                   // [P] gradient of the current field
-    float *xs = gacc + round4(P);                         // [128][XS]
-    float *dzs = xs + kThreads * XS;                      // [128][DS]
-    const int tid = threadIdx.x;
-    float *xrow = xs + tid * XS;
-    float *drow = dzs + tid * DS;
-
-    for (int q = tid; q < P; q += kThreads) gacc[q] = 0.f;
+    using F = FbShape<W, H>;
+    constexpr int S = F::S, XS = F::XS, KC = F::KC, NST = F::kStages;
+    constexpr ALayout A(W, H);
+    constexpr RLayout RL(W, H);
+    constexpr TLayout TL(W, H);
+    extern __shared__ float4 smem4[];
+    __shared__ int2 entries[F::kPer];      // a tile's ring stages: offset in wt (or -1 - offset in wr), 16-byte pieces
+    float *X = reinterpret_cast<float *>(smem4);
+    float *ring = X + F::kRows * XS;
+    float *tab = ring + NST * F::kStage;
+    float *dzo = tab + F::kTab;                       // [3][S] d loss / d output logit, then [S] of the density's
+    float *gacc = dzo + 4 * S;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int q = tid; q < F::kGrad; q += kThreads) gacc[q] = 0.f;
+    // the order in which a tile reads its weight rows
+    for (int e = tid; e < F::kPer; e += kThreads) {
+        int at = 0;
+        int2 en = make_int2(0, 0);
+        auto piece = [&](int64_t off, bool dgrad, int n_rows, int ld) {
+            const int n = (n_rows + kRingRows - 1) / kRingRows, r = e - at;
+            at += n;
+            if (r < 0 || r >= n) return;
+            const int o = (int)off + r * kRingRows * ld;
+            en = make_int2(dgrad ? -1 - o : o, min(kRingRows, n_rows - r * kRingRows) * ld / 4);
+        };
+        piece(TL.l1, false, kPeX, W);
+        for (int l = 1; l < H; ++l) piece(TL.hid + (int64_t)(l - 1) * (W * W + W), false, W, W);
+        piece(TL.head, false, W, F::NH);
+        piece(TL.col, false, KC, W);
+        piece(RL.col, true, W, W);
+        piece(RL.head, true, W, W);
+        for (int l = H - 1; l >= 1; --l) piece(RL.hid + (int64_t)(l - 1) * W * W, true, W, W);
+        entries[e] = en;
+    }
     __syncthreads();
+
     const uint32_t n_tiles = ctr->n_tiles;
     const uint32_t t0 = (uint32_t)((uint64_t)n_tiles * blockIdx.x / gridDim.x);
     const uint32_t t1 = (uint32_t)((uint64_t)n_tiles * (blockIdx.x + 1) / gridDim.x);
-    uint32_t cur = 0xffffffffu;
-    for (uint32_t t = t0; t <= t1; ++t) {
-        const uint32_t f = t < t1 ? b.tiles[t].field : 0xfffffffeu;
-        if (f != cur) {
-            if (cur != 0xffffffffu) {
-                float *gf = grad + (int64_t)cur * w.P;
-                for (int q = tid; q < P; q += kThreads) {
-                    const float v = gacc[q];
-                    if (v != 0.f) atomicAdd(gf + q, v);
-                    gacc[q] = 0.f;
-                }
-                __syncthreads();
-            }
-            cur = f;
-        }
-        if (t == t1) break;
-        const Tile tl = b.tiles[t];
-        const bool valid = (uint32_t)tid < tl.count;
-        const uint32_t idx = valid ? b.sorted[tl.start + tid] : 0u;
-        const float *aff = w.affine + 6 * (int64_t)tl.field;
-        float xl0 = 0.f, xl1 = 0.f, xl2 = 0.f, dx = 0.f, dy = 0.f, dz = 1.f;
-        float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (valid && src.mode == 1) {
-            // direct points (distillation): world position and direction per sample
-            const float px = src.p[3 * (int64_t)idx], py = src.p[3 * (int64_t)idx + 1], pz = src.p[3 * (int64_t)idx + 2];
-            dx = src.d[3 * (int64_t)idx]; dy = src.d[3 * (int64_t)idx + 1]; dz = src.d[3 * (int64_t)idx + 2];
-            xl0 = fmaf(aff[0], px, aff[3]);
-            xl1 = fmaf(aff[1], py, aff[4]);
-            xl2 = fmaf(aff[2], pz, aff[5]);
-            g = gsr[idx];
-        } else if (valid) {
-            const uint32_t col = idx >> 5;
-            const uint32_t i = (col / (uint32_t)src.R) * 32u + (idx & 31u);
-            const uint32_t ray = src.live ? src.live[i] : i;
-            const uint32_t j = src.recs[idx] & 0xffffu;
-            const float4 o = src.st.orig[ray], d = src.st.dir[ray];
-            dx = d.x; dy = d.y; dz = d.z;
-            if (src.accurate) {
-                const float4 dl = src.st.dir_lo[ray];
-                const float th0 = (float)j + 0.5f;
-                xl0 = local_coord(th0, src.delta, o.x, d.x, dl.x, aff[0], aff[3]);
-                xl1 = local_coord(th0, src.delta, o.y, d.y, dl.y, aff[1], aff[4]);
-                xl2 = local_coord(th0, src.delta, o.z, d.z, dl.z, aff[2], aff[5]);
-            } else {
-                const float tt = ((float)j + 0.5f) * src.delta;
-                xl0 = fmaf(aff[0], fmaf(tt, d.x, o.x), aff[3]);
-                xl1 = fmaf(aff[1], fmaf(tt, d.y, o.y), aff[4]);
-                xl2 = fmaf(aff[2], fmaf(tt, d.z, o.z), aff[5]);
-            }
-            g = gsr[idx];
-        }
-        const float *wtf = w.wt + (int64_t)tl.field * w.Pt;
-        const float *wrf = w.wr + (int64_t)tl.field * w.Pr;
-        float *gf = gacc;
 
-        // ---- forward recompute, activations kept per thread ----
-        float pe[kPeX];
-        encode_arr<10>(xl0, xl1, xl2, pe);
-        float hs[H][W];
-        {
-            float acc[W];
-            dense_arr<kPeX, W>(pe, wtf + TL.l1, acc);
-#pragma unroll
-            for (int o = 0; o < W; ++o) hs[0][o] = fmaxf(acc[o], 0.f);
-        }
-#pragma unroll
-        for (int l = 1; l < H; ++l) {
-            float acc[W];
-            dense_arr<W, W>(hs[l - 1], wtf + TL.hid + (int64_t)(l - 1) * (W * W + W), acc);
-#pragma unroll
-            for (int o = 0; o < W; ++o) hs[l][o] = fmaxf(acc[o], 0.f);
-        }
-        float inc[KC];                    // [features; F(d)]
-        float s_logit;
-        {
-            float acc[NH];
-            dense_arr<W, NH>(hs[H - 1], wtf + TL.head, acc);
-            s_logit = acc[W];             // the transposed head: features, then the density logit
-#pragma unroll
-            for (int o = 0; o < W; ++o) inc[o] = acc[o];
-        }
-        encode_arr<4>(dx, dy, dz, inc + W);
-        float gg[W];
-        {
-            float acc[W];
-            dense_arr<KC, W>(inc, wtf + TL.col, acc);
-#pragma unroll
-            for (int o = 0; o < W; ++o) gg[o] = fmaxf(acc[o], 0.f);
-        }
-        float rgb[3];
-        {
-            float acc[4];
-            dense_arr<W, 4>(gg, wtf + TL.out, acc);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) rgb[c] = 1.f / (1.f + expf(-acc[c]));
-        }
-
-        // ---- output layer: rgb = sigmoid(zo) ----
-        float dzo[3] = {g.y * rgb[0] * (1.f - rgb[0]), g.z * rgb[1] * (1.f - rgb[1]), g.w * rgb[2] * (1.f - rgb[2])};
-        stage_row(xrow, gg, W);
-        stage_row(drow, dzo, 3);
-        __syncthreads();
-        wgrad<3, W, XS, DS>(xs, dzs, gf + A.out, gf + A.out + 3 * W, tid);
-        float dv[round4(KC)];
-        {
-            float d_g[W];
-            dgrad<3, W>(drow, wrf + RL.out, d_g);
-#pragma unroll
-            for (int k = 0; k < W; ++k) dv[k] = gg[k] > 0.f ? d_g[k] : 0.f;
-        }
-        __syncthreads();
-        // ---- colour layer: g = relu(Wc [feat; F(d)] + bc) ----
-        stage_row(xrow, inc, KC);
-        {
-            float t[W];
-#pragma unroll
-            for (int k = 0; k < W; ++k) t[k] = dv[k];
-            stage_row(drow, t, W);
-        }
-        __syncthreads();
-        wgrad<W, KC, XS, DS>(xs, dzs, gf + A.col, gf + A.col + (int64_t)W * KC, tid);
-        {
-            float d_in[round4(KC)];
-            dgrad<W, round4(KC)>(drow, wrf + RL.col, d_in);
-#pragma unroll
-            for (int k = 0; k < W; ++k) dv[k] = d_in[k];       // d feat (features have no activation)
-        }
-        __syncthreads();
-        // ---- head: [s; feat] = Wh h_H + bh, sigma = scale * softplus(s) ----
-        {
-            const float ds = g.x * w.sigma_scale *
-                             (w.act == ROAM_RELU ? (s_logit > 0.f ? 1.f : 0.f) : 1.f / (1.f + expf(-s_logit)));
-            float t[W + 1];
-            t[0] = ds;
-#pragma unroll
-            for (int k = 0; k < W; ++k) t[1 + k] = dv[k];
-            stage_row(xrow, hs[H - 1], W);
-            stage_row(drow, t, W + 1);
-        }
-        __syncthreads();
-        wgrad<W + 1, W, XS, DS>(xs, dzs, gf + A.head, gf + A.head + (int64_t)(1 + W) * W, tid);
-        {
-            float d_h[W];
-            dgrad<W + 1, W>(drow, wrf + RL.head, d_h);
-#pragma unroll
-            for (int k = 0; k < W; ++k) dv[k] = hs[H - 1][k] > 0.f ? d_h[k] : 0.f;
-        }
-        __syncthreads();
-        // ---- hidden layers H..2 ----
-#pragma unroll
-        for (int l = H - 1; l >= 1; --l) {
-            {
-                float t[W];
-#pragma unroll
-                for (int k = 0; k < W; ++k) t[k] = dv[k];
-                stage_row(xrow, hs[l - 1], W);
-                stage_row(drow, t, W);
+    Tile tl{0u, 0u, 0u, 0u};                        // the next tile
+    // the ring's feed, by warps 0-3: stage j of the run is entry j mod kPer of
+    // its tile's list, into slot j mod NST
+    uint32_t issue_s = 0, issue_e = 0, issue_t = t0, issue_f = 0u;
+    auto feed = [&]() {
+        if (issue_t < t1) {
+            const int2 en = entries[issue_e];
+            const float *rows = en.x >= 0 ? w.wt + (int64_t)issue_f * w.Pt + en.x : w.wr + (int64_t)issue_f * w.Pr + (-1 - en.x);
+            float *dst = ring + issue_s * F::kStage;
+            for (int c = tid; c < en.y; c += 128) cp_async16(dst + 4 * c, rows + 4 * c);
+            if (++issue_s == (uint32_t)NST) issue_s = 0;
+            if (++issue_e == (uint32_t)F::kPer) {
+                issue_e = 0;
+                ++issue_t;
+                issue_f = tl.field;                 // (a tile has more entries than the ring has stages)
             }
-            __syncthreads();
-            const int64_t ob = A.hid + (int64_t)(l - 1) * (W * W + W);
-            wgrad<W, W, XS, DS>(xs, dzs, gf + ob, gf + ob + (int64_t)W * W, tid);
-            {
-                float d_h[W];
-                dgrad<W, W>(drow, wrf + RL.hid + (int64_t)(l - 1) * W * W, d_h);
-#pragma unroll
-                for (int k = 0; k < W; ++k) dv[k] = hs[l - 1][k] > 0.f ? d_h[k] : 0.f;
-            }
-            __syncthreads();
         }
-        // ---- layer 1 ----
-        {
-            float t[W];
-#pragma unroll
-            for (int k = 0; k < W; ++k) t[k] = dv[k];
-            stage_row(xrow, pe, kPeX);
-            stage_row(drow, t, W);
-        }
-        __syncthreads();
-        wgrad<W, kPeX, XS, DS>(xs, dzs, gf + A.l1, gf + A.l1 + (int64_t)W * kPeX, tid);
-        __syncthreads();
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (warp < 4 && t0 < t1) {
+        issue_f = b.tiles[t0].field;
+#pragma unroll 1
+        for (int j = 0; j + 1 < NST; ++j) feed();
     }
+
+    // forward and dgrad: a warp covers 32 samples x 4 TN (TD) outputs, lane =
+    // 8 sample groups of 4 x 4 output groups
+    constexpr int SB = S / 32;
+    const int sg = lane & 7, og = lane >> 3;
+    const int sF = (warp % SB) * 32 + 4 * sg;                       // first sample
+    const int nF = (warp / SB) * 4 * F::TN + og * F::TN;            // first forward output
+    const int kD = ((warp & 3) / SB) * 4 * F::TD + og * F::TD;      // first dgrad input (warps 0-3)
+    uint32_t slot = 0;                                              // ring slot of the next stage to consume
+    auto sync = [&]() { bar_sync(1, kThreads); };
+
+    // acc[s][j] += sum over the next K ring rows of x[k][sF + s] row[col + j]
+    // (by TH threads: all, or warps 0-3)
+    auto dense = [&](auto KK, auto LDc, auto TT, auto THc, const float *x, int col,
+                     float2 (&acc)[4][decltype(TT)::value / 2]) {
+        constexpr int K = decltype(KK)::value, LD = decltype(LDc)::value, T = decltype(TT)::value,
+                      TH = decltype(THc)::value;
+        auto rows = [&](auto NR, int k0) {
+            // the stage has landed for every loader, and every consumer is past
+            // the stage before it, whose slot takes the next copy
+            if (warp < 4) cp_async_wait<NST - 2>();
+            bar_sync(TH == 256 ? 1 : 2, TH);
+            if (warp < 4) feed();
+            const float *wrow = ring + slot * F::kStage + col;
+            const float *xr = x + (int64_t)k0 * XS + sF;
+#pragma unroll
+            for (int kk = 0; kk < decltype(NR)::value; ++kk) {
+                float2 wv[T / 2];
+                ld_row<T>(wrow + kk * LD, wv);
+                const float4 xv = *reinterpret_cast<const float4 *>(xr + kk * XS);
+                const float2 xx[4] = {make_float2(xv.x, xv.x), make_float2(xv.y, xv.y), make_float2(xv.z, xv.z),
+                                      make_float2(xv.w, xv.w)};
+#pragma unroll
+                for (int j = 0; j < T / 2; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) acc[q][j] = __ffma2_rn(wv[j], xx[q], acc[q][j]);
+            }
+            if (++slot == (uint32_t)NST) slot = 0;
+        };
+#pragma unroll 1
+        for (int k0 = 0; k0 + kRingRows <= K; k0 += kRingRows) rows(Int<kRingRows>{}, k0);
+        if constexpr (K % kRingRows != 0) rows(Int<K % kRingRows>{}, K - K % kRingRows);
+    };
+    // rows r .. of the activations from this thread's outputs, 4 samples at once
+    auto store = [&](auto TT, float *row, const float2 (&acc)[4][decltype(TT)::value / 2], bool relu) {
+#pragma unroll
+        for (int j = 0; j < decltype(TT)::value; ++j) {
+            float4 v = (j & 1) ? make_float4(acc[0][j / 2].y, acc[1][j / 2].y, acc[2][j / 2].y, acc[3][j / 2].y)
+                               : make_float4(acc[0][j / 2].x, acc[1][j / 2].x, acc[2][j / 2].x, acc[3][j / 2].x);
+            if (relu) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+            *reinterpret_cast<float4 *>(row + j * XS + sF) = v;
+        }
+    };
+    // this tile's wgrad of one layer by kW warps (wi = this warp's index among
+    // them): g[n][k] += sum_s dz[n][s] x[k][s]; a lane owns outputs
+    // ln + 8 i and inputs kb + lk + 4 j, so a warp covers W x 4 TK
+    auto wgrad = [&](auto KK, auto KW, int wi, const float *dz, const float *x, float *g, int ldg) {
+        constexpr int K = decltype(KK)::value, TNW = W / 8;
+        constexpr int TK = (K + 4 * decltype(KW)::value - 1) / (4 * decltype(KW)::value);
+        const int ln = lane & 7, lk = lane >> 3, kb = wi * 4 * TK + lk;
+        float2 acc[TNW][TK];
+#pragma unroll
+        for (int i = 0; i < TNW; ++i)
+#pragma unroll
+            for (int j = 0; j < TK; ++j) acc[i][j] = make_float2(0.f, 0.f);
+        const float *dzr = dz + ln * XS;
+        const float *xr[TK];
+#pragma unroll
+        for (int j = 0; j < TK; ++j) xr[j] = x + min(kb + 4 * j, K - 1) * XS;    // (rows past K: computed, not kept)
+#pragma unroll 2
+        for (int s = 0; s < S; s += 4) {
+            float4 xv[TK];
+#pragma unroll
+            for (int j = 0; j < TK; ++j) xv[j] = *reinterpret_cast<const float4 *>(xr[j] + s);
+#pragma unroll
+            for (int i = 0; i < TNW; ++i) {
+                const float4 d = *reinterpret_cast<const float4 *>(dzr + 8 * i * XS + s);
+#pragma unroll
+                for (int j = 0; j < TK; ++j) {
+                    acc[i][j] = __ffma2_rn(make_float2(d.x, d.y), make_float2(xv[j].x, xv[j].y), acc[i][j]);
+                    acc[i][j] = __ffma2_rn(make_float2(d.z, d.w), make_float2(xv[j].z, xv[j].w), acc[i][j]);
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < TK; ++j) {
+            const int k = kb + 4 * j;
+            if (k >= K) continue;
+#pragma unroll
+            for (int i = 0; i < TNW; ++i) g[(ln + 8 * i) * ldg + k] += acc[i][j].x + acc[i][j].y;
+        }
+    };
+    // row sums over the samples: out[n] += sum_s v[n][s] m[s] (m may be null: 1),
+    // n < W, by the 128 threads of a half (ht = thread within it)
+    auto row_sums = [&](int ht, const float *v, const float *m, float *out) {
+        constexpr int PT = 128 / W;
+        const int n = ht / PT, p = ht % PT;
+        float a = 0.f;
+#pragma unroll 4
+        for (int s = 4 * p; s < S; s += 4 * PT) {
+            const float4 q = *reinterpret_cast<const float4 *>(v + n * XS + s);
+            if (m) {
+                const float4 e = *reinterpret_cast<const float4 *>(m + s);
+                a = fmaf(q.x, e.x, a);
+                a = fmaf(q.y, e.y, a);
+                a = fmaf(q.z, e.z, a);
+                a = fmaf(q.w, e.w, a);
+            } else {
+                a += (q.x + q.y) + (q.z + q.w);
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < PT; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (p == 0) out[n] += a;
+    };
+    // the accumulated gradient of field f to global memory, and cleared
+    auto flush_part = [&](float *gf, float *rows, int n_out, int n_in, int ld) {
+#pragma unroll 4
+        for (int n = warp; n < n_out; n += 8) {
+#pragma unroll 3
+            for (int k = lane; k < n_in; k += 32) {
+                const float v = rows[n * ld + k];
+                if (v != 0.f) atomicAdd(gf + n * n_in + k, v);
+                rows[n * ld + k] = 0.f;
+            }
+        }
+    };
+    auto flush = [&](uint32_t f) {
+        float *gf = grad + (int64_t)f * w.P;
+        flush_part(gf + A.l1, gacc + F::gA, W, kPeX, F::SA);
+        flush_part(gf + A.l1 + W * kPeX, gacc + F::gB, 1, W, W);
+        for (int l = 1; l < H; ++l) {
+            const int64_t o = A.hid + (int64_t)(l - 1) * (W * W + W);
+            flush_part(gf + o, gacc + F::gHid + (l - 1) * W * F::SH, W, W, F::SH);
+            flush_part(gf + o + W * W, gacc + F::gB + l * W, 1, W, W);
+        }
+        flush_part(gf + A.head, gacc + F::gDen, 1, W, W);
+        flush_part(gf + A.head + W, gacc + F::gHead, W, W, F::SH);
+        flush_part(gf + A.head + (1 + W) * W, gacc + F::gBd, 1, 1, 1);
+        flush_part(gf + A.head + (1 + W) * W + 1, gacc + F::gB + H * W, 1, W, W);
+        flush_part(gf + A.col, gacc + F::gCol, W, KC, F::SC);
+        flush_part(gf + A.col + W * KC, gacc + F::gB + (H + 1) * W, 1, W, W);
+        flush_part(gf + A.out, gacc + F::gOut, 3, W, W);
+        flush_part(gf + A.out + 3 * W, gacc + F::gBd + 1, 1, 3, 3);
+    };
+
+    uint32_t cur = 0xffffffffu;
+    const int smp = tid % S;                     // this thread's sample in the gather and the encoding
+    constexpr int NP = kThreads / S;             // threads per sample
+    const int part = tid / S;
+    FbPending pend{};
+    if (t0 < t1) {
+        tl = b.tiles[t0];
+        fb_index(pend, b, tl, smp, true);
+        fb_record(pend, src);
+        fb_ray(pend, src);
+    }
+    for (uint32_t t = t0; t < t1; ++t) {
+        const Tile tc = tl;
+        const FbPending me = pend;
+        const bool more = t + 1 < t1;
+        if (more) tl = b.tiles[t + 1];
+        // (every thread is past the previous tile's last reads: the barrier below)
+        sync();
+        if (tc.field != cur) {
+            if (cur != 0xffffffffu) flush(cur);
+            cur = tc.field;
+            const float *wf = w.w32 + (int64_t)cur * w.P;
+            for (int q = tid; q < F::kTab; q += kThreads) {
+                float v = 0.f;
+                if (q < F::tDen) {
+                    const int l = q / W, n = q % W;
+                    v = l == 0 ? wf[A.l1 + W * kPeX + n]
+                               : (l < H ? wf[A.hid + (int64_t)(l - 1) * (W * W + W) + W * W + n]
+                                        : (l == H ? wf[A.head + (1 + W) * W + 1 + n] : wf[A.col + W * KC + n]));
+                } else if (q < F::tOut) v = wf[A.head + (q - F::tDen)];
+                else if (q < F::tBd) v = wf[A.out + (q - F::tOut)];
+                else if (q == F::tBd) v = wf[A.head + (1 + W) * W];
+                else if (q < F::tBd + 4) v = wf[A.out + 3 * W + (q - F::tBd - 1)];
+                tab[q] = v;
+            }
+        }
+        // ---- encode: the sample's frequencies split over its NP threads ----
+        const float4 gv = me.on ? gsr[me.idx] : make_float4(0.f, 0.f, 0.f, 0.f);
+        {
+            const float *aff = w.affine + 6 * (int64_t)tc.field;
+            float xl[3] = {0.f, 0.f, 0.f}, dv[3] = {0.f, 0.f, 1.f};
+            if (me.on) {
+                const float op[3] = {me.o.x, me.o.y, me.o.z}, dp[3] = {me.d.x, me.d.y, me.d.z},
+                            lp[3] = {me.dl.x, me.dl.y, me.dl.z};
+                const float th0 = (float)(me.rec & 0xffffu) + 0.5f;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    dv[a] = dp[a];
+                    if (src.mode == 1) xl[a] = fmaf(aff[a], op[a], aff[3 + a]);
+                    else if (src.accurate) xl[a] = local_coord(th0, src.delta, op[a], dp[a], lp[a], aff[a], aff[3 + a]);
+                    else xl[a] = fmaf(aff[a], fmaf(th0 * src.delta, dp[a], op[a]), aff[3 + a]);
+                }
+            }
+            float *xp = X + F::rX * XS + smp, *dp = X + (F::rC + W) * XS + smp;
+            if (part == 0) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) xp[a * XS] = xl[a];
+            } else if (part == 1) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) dp[a * XS] = dv[a];
+            }
+            for (int k = part; k < 14; k += NP) {
+                const bool pos = k < 10;
+                const int kk = pos ? k : k - 10;
+                float *row = (pos ? xp : dp) + (3 + 6 * kk) * XS;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    float s, c;
+                    sincospif(ldexpf(pos ? xl[a] : dv[a], kk), &s, &c);
+                    row[a * XS] = s;
+                    row[(3 + a) * XS] = c;
+                }
+            }
+        }
+        sync();
+
+        // ---- forward recompute ----
+        auto forward = [&](auto KK, auto LDc, int layer, const float *x, float *y, bool relu) {
+            float2 acc[4][F::TN / 2];
+#pragma unroll
+            for (int j = 0; j < F::TN / 2; ++j) {
+                const float2 bb = *reinterpret_cast<const float2 *>(tab + F::tB + layer * W + nF + 2 * j);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[q][j] = bb;
+            }
+            dense(KK, LDc, Int<F::TN>{}, Int<256>{}, x, nF, acc);
+            store(Int<F::TN>{}, y + nF * XS, acc, relu);
+            sync();
+        };
+        forward(Int<kPeX>{}, Int<W>{}, 0, X + F::rX * XS, X + F::rH(1) * XS, true);
+        fb_index(pend, b, tl, smp, more);
+#pragma unroll 1
+        for (int l = 1; l < H; ++l)
+            forward(Int<W>{}, Int<W>{}, l, X + F::rH(l) * XS, X + F::rH(l + 1) * XS, true);
+        forward(Int<W>{}, Int<F::NH>{}, H, X + F::rH(H) * XS, X + F::rC * XS, false);
+        fb_record(pend, src);
+        forward(Int<KC>{}, Int<W>{}, H + 1, X + F::rC * XS, X + F::rG * XS, true);
+        fb_ray(pend, src);
+
+        // ---- outputs and the loss gradient at their logits: rgb by parts
+        // 0 .. 2, the density by part 3 (a sample's parts go round its threads) ----
+#pragma unroll 1
+        for (int e = part; e < 4; e += NP) {
+            const float *row = (e < 3 ? X + F::rG * XS : X + F::rH(H) * XS) + smp;
+            const float *wv = tab + (e < 3 ? F::tOut + e * W : F::tDen);
+            float z = tab[F::tBd + (e < 3 ? 1 + e : 0)];
+#pragma unroll 16
+            for (int k = 0; k < W; ++k) z = fmaf(wv[k], row[k * XS], z);
+            if (e < 3) {
+                const float c = 1.f / (1.f + expf(-z));
+                dzo[e * S + smp] = (e == 0 ? gv.y : (e == 1 ? gv.z : gv.w)) * c * (1.f - c);
+            } else {
+                dzo[3 * S + smp] = gv.x * w.sigma_scale *
+                                   (w.act == ROAM_RELU ? (z > 0.f ? 1.f : 0.f) : 1.f / (1.f + expf(-z)));
+            }
+        }
+        sync();
+
+        // ---- output layer: its wgrad, and dZ of the colour layer in g's place ----
+        {
+            constexpr int PT = kThreads / W;
+            const int n = tid / PT, p = tid % PT;
+            const float w0 = tab[F::tOut + n], w1 = tab[F::tOut + W + n], w2 = tab[F::tOut + 2 * W + n];
+            float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+#pragma unroll 2
+            for (int s = 4 * p; s < S; s += 4 * PT) {
+                float4 *gp = reinterpret_cast<float4 *>(X + (F::rG + n) * XS + s);
+                const float4 g4 = *gp;
+                const float4 z0 = *reinterpret_cast<const float4 *>(dzo + s),
+                             z1 = *reinterpret_cast<const float4 *>(dzo + S + s),
+                             z2 = *reinterpret_cast<const float4 *>(dzo + 2 * S + s);
+                const float gg[4] = {g4.x, g4.y, g4.z, g4.w}, y0[4] = {z0.x, z0.y, z0.z, z0.w},
+                            y1[4] = {z1.x, z1.y, z1.z, z1.w}, y2[4] = {z2.x, z2.y, z2.z, z2.w};
+                float dz[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    a0 = fmaf(y0[q], gg[q], a0);
+                    a1 = fmaf(y1[q], gg[q], a1);
+                    a2 = fmaf(y2[q], gg[q], a2);
+                    const float d = fmaf(w2, y2[q], fmaf(w1, y1[q], w0 * y0[q]));
+                    dz[q] = gg[q] > 0.f ? d : 0.f;
+                }
+                *gp = make_float4(dz[0], dz[1], dz[2], dz[3]);
+            }
+#pragma unroll
+            for (int o = 1; o < PT; o <<= 1) {
+                a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+                a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+                a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+            }
+            if (p == 0) {
+                gacc[F::gOut + n] += a0;
+                gacc[F::gOut + W + n] += a1;
+                gacc[F::gOut + 2 * W + n] += a2;
+            }
+            if (warp < 4) {
+                // the output biases (warps 0-2) and the density's (warp 3)
+                float a = 0.f;
+#pragma unroll
+                for (int s = lane; s < S; s += 32) a += dzo[warp * S + s];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                if (lane == 0) gacc[F::gBd + (warp == 3 ? 0 : 1 + warp)] += a;
+            }
+        }
+        sync();
+
+        // ---- colour, head and hidden layers: dgrad by warps 0-3 beside
+        // wgrad by warps 4-7; then dX, masked, over the layer's input ----
+        auto backward = [&](auto KK, int layer, const float *dz, float *x, float *g, int ldg, int kind) {
+            float2 acc[4][F::TD / 2];
+            if (warp < 4) {
+                // the head's density row first (kind 1), as the layer's output 0
+#pragma unroll
+                for (int j = 0; j < F::TD / 2; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) acc[q][j] = make_float2(0.f, 0.f);
+                if (kind == 1) {
+                    float2 wv[F::TD / 2];
+                    ld_row<F::TD>(tab + F::tDen + kD, wv);
+                    const float4 d = *reinterpret_cast<const float4 *>(dzo + 3 * S + sF);
+                    const float dd[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+                    for (int j = 0; j < F::TD / 2; ++j)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) acc[q][j] = make_float2(wv[j].x * dd[q], wv[j].y * dd[q]);
+                }
+                dense(Int<W>{}, Int<W>{}, Int<F::TD>{}, Int<128>{}, dz, kD, acc);
+                row_sums(tid, dz, nullptr, gacc + F::gB + layer * W);
+                if (kind == 1) row_sums(tid, x, dzo + 3 * S, gacc + F::gDen);
+            } else {
+                wgrad(KK, Int<4>{}, warp - 4, dz, x, g, ldg);
+                slot = (slot + W / kRingRows) % NST;
+            }
+            sync();
+            if (warp < 4) {
+                if (kind != 0) {
+#pragma unroll
+                    for (int j = 0; j < F::TD; ++j) {
+                        const float4 h = *reinterpret_cast<const float4 *>(x + (kD + j) * XS + sF);
+                        float *c[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) c[q] = (j & 1) ? &acc[q][j / 2].y : &acc[q][j / 2].x;
+                        if (!(h.x > 0.f)) *c[0] = 0.f;
+                        if (!(h.y > 0.f)) *c[1] = 0.f;
+                        if (!(h.z > 0.f)) *c[2] = 0.f;
+                        if (!(h.w > 0.f)) *c[3] = 0.f;
+                    }
+                }
+                store(Int<F::TD>{}, x + kD * XS, acc, false);
+            }
+            sync();
+        };
+        // (kind 0: the features carry no activation)
+        backward(Int<KC>{}, H + 1, X + F::rG * XS, X + F::rC * XS, gacc + F::gCol, F::SC, 0);
+        backward(Int<W>{}, H, X + F::rC * XS, X + F::rH(H) * XS, gacc + F::gHead, F::SH, 1);
+#pragma unroll 1
+        for (int l = H - 1; l >= 1; --l)
+            backward(Int<W>{}, l, X + F::rH(l + 1) * XS, X + F::rH(l) * XS,
+                            gacc + F::gHid + (l - 1) * W * F::SH, F::SH, 2);
+        // ---- layer 1: wgrad only, by every warp ----
+        wgrad(Int<kPeX>{}, Int<8>{}, warp, X + F::rH(1) * XS, X + F::rX * XS, gacc + F::gA, F::SA);
+        if (warp < 4) row_sums(tid, X + F::rH(1) * XS, nullptr, gacc + F::gB);
+    }
+    sync();
+    if (cur != 0xffffffffu) flush(cur);
 }
 
-// API layout -> row-padded copy (matrices only)
+// API layout -> the dgrad copy (matrices only)
 __global__ void k_pack_rows(const float *__restrict__ w32, int n_fields, int W, int H, int64_t P,
                             float *__restrict__ wr, int64_t Pr)
 {
     const ALayout A(W, H);
     const RLayout RL(W, H);
-    const int64_t n = (int64_t)n_fields * P;
-    for (int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gidx < n;
-         gidx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t f = gidx / P, q = gidx % P;
-        int64_t src0, dst0;
-        int n_out, n_in, kp;
-        if (q < A.hid) { src0 = A.l1; dst0 = RL.l1; n_out = W; n_in = kPeX; }
-        else if (q < A.head) {
-            const int64_t l = (q - A.hid) / ((int64_t)W * W + W);
-            src0 = A.hid + l * (W * W + W); dst0 = RL.hid + l * W * W; n_out = W; n_in = W;
-        }
-        else if (q < A.col) { src0 = A.head; dst0 = RL.head; n_out = 1 + W; n_in = W; }
-        else if (q < A.out) { src0 = A.col; dst0 = RL.col; n_out = W; n_in = W + kPeD; }
-        else { src0 = A.out; dst0 = RL.out; n_out = 3; n_in = W; }
-        kp = round4(n_in);
-        const int64_t r = q - src0;
-        if (r >= (int64_t)n_out * n_in) continue;      // a bias
-        const int64_t o = r / n_in, i = r % n_in;
-        wr[f * Pr + dst0 + o * kp + i] = w32[gidx];
+    const int f = blockIdx.y;
+    const float *wf = w32 + (int64_t)f * P;
+    float *df = wr + (int64_t)f * Pr;
+    for (int q = (int)(blockIdx.x * blockDim.x + threadIdx.x); q < (int)Pr; q += (int)(gridDim.x * blockDim.x)) {
+        const int m = q / (W * W), r = q - m * W * W;
+        int64_t s;
+        if (m < H - 1) s = A.hid + (int64_t)m * (W * W + W) + r;
+        else if (m == H - 1) s = A.head + W + r;                                  // past the density row
+        else s = A.col + (int64_t)(r / W) * (W + kPeD) + r % W;
+        df[q] = wf[s];
     }
 }
 
@@ -458,14 +708,14 @@ template <int W, int H>
 void launch_bwd_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, const float4 *gsr,
                   float *grad, int grid, cudaStream_t s)
 {
-    constexpr int KC = W + kPeD;
-    constexpr int KMAX = KC > kPeX ? KC : kPeX;
-    const size_t sh = ((size_t)round4((int)ALayout(W, H).total) + (size_t)kThreads * (KMAX + 1) +
-                       (size_t)kThreads * (W + 2)) * sizeof(float);
     static int smem_set[kMaxDevices] = {};
-    raise_smem_limit((const void *)k_mlp_bwd_simt<W, H>, (int)sh, smem_set);
-    k_mlp_bwd_simt<W, H><<<grid, kThreads, sh, s>>>(w, src, b, ctr, gsr, grad);
+    raise_smem_limit((const void *)k_mlp_bwd_simt<W, H>, (int)FbShape<W, H>::kSmem, smem_set);
+    k_mlp_bwd_simt<W, H><<<grid, kThreads, FbShape<W, H>::kSmem, s>>>(w, src, b, ctr, gsr, grad);
 }
+
+#define ROAM_FB_CASES                                                          \
+    ROAM_CASE(32, 1) ROAM_CASE(32, 2) ROAM_CASE(32, 3) ROAM_CASE(32, 4) \
+    ROAM_CASE(64, 1) ROAM_CASE(64, 2) ROAM_CASE(64, 3) ROAM_CASE(64, 4)
 
 }  // namespace
 
@@ -473,10 +723,18 @@ bool mlp_bwd_supported(int W, int H) { return (W == 32 || W == 64) && H >= 1 && 
 
 int64_t rows_padded_size(int W, int H) { return RLayout(W, H).total; }
 
+int mlp_bwd_simt_tile(int W, int H)
+{
+#define ROAM_CASE(WW, HH) \
+    if (W == WW && H == HH) return FbShape<WW, HH>::S;
+    ROAM_FB_CASES
+#undef ROAM_CASE
+    return 128;
+}
+
 void launch_pack_rows(const float *w32, int n_fields, int W, int H, int64_t P, float *wr, int64_t Pr, cudaStream_t s)
 {
-    cudaMemsetAsync(wr, 0, (size_t)n_fields * Pr * sizeof(float), s);
-    k_pack_rows<<<1024, 256, 0, s>>>(w32, n_fields, W, H, P, wr, Pr);
+    k_pack_rows<<<dim3((unsigned)((Pr + 1023) / 1024), (unsigned)n_fields), 256, 0, s>>>(w32, n_fields, W, H, P, wr, Pr);
 }
 
 void launch_mlp_bwd_simt(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr,
@@ -484,8 +742,7 @@ void launch_mlp_bwd_simt(const MlpWeights &w, const SampleSrc &src, const Bucket
 {
 #define ROAM_CASE(WW, HH) \
     if (w.W == WW && w.H == HH) { launch_bwd_t<WW, HH>(w, src, b, ctr, gsr, grad, grid, s); return; }
-    ROAM_CASE(32, 1) ROAM_CASE(32, 2) ROAM_CASE(32, 3) ROAM_CASE(32, 4)
-    ROAM_CASE(64, 1) ROAM_CASE(64, 2) ROAM_CASE(64, 3) ROAM_CASE(64, 4)
+    ROAM_FB_CASES
 #undef ROAM_CASE
 }
 

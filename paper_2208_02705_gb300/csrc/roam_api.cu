@@ -416,13 +416,12 @@ roam_status upload_cams(roam_ctx *c, const roam_camera *cams, int n_views, float
     return ROAM_OK;
 }
 
-// tile records needed for `samples` samples: one per 128 plus padding of
-// each field's run to a whole group
-// tiles of 128 samples, each field's run rounded up to its padding (at most
-// the larger of 8 and the forced padding)
-size_t tile_capacity(const roam_ctx *c, size_t samples)
+// tile records needed for `samples` samples in tiles of `tile`: each field's
+// run rounded up to its padding (at most the larger of 8 and the forced
+// padding)
+size_t tile_capacity(const roam_ctx *c, size_t samples, int tile = 128)
 {
-    return samples / 128 + (size_t)c->n_fields * (size_t)std::max(8, c->tile_pad) + 1;
+    return samples / (size_t)tile + (size_t)c->n_fields * (size_t)std::max(8, c->tile_pad) + 1;
 }
 
 roam_status ensure_rays(roam_ctx *c, int64_t n_rays, int R)
@@ -1319,11 +1318,12 @@ roam_status roam_mlp_backward(roam_ctx *c, const float *p, const float *d, const
     if (n == 0) return ROAM_OK;
     if (!p || !d || !field || !dl_dout) return fail(ROAM_ERR_ARG, "null pointer");
     if (((uintptr_t)dl_dout) & 15) return fail(ROAM_ERR_ARG, "dl_dout must be 16-byte aligned");
+    const int tile = tc ? 128 : mlp_bwd_simt_tile(c->md.width, c->md.n_hidden);
     ROAM_TRY(ensure(c->sorted, (size_t)n));
-    ROAM_TRY(ensure(c->tiles, tile_capacity(c, (size_t)n)));
+    ROAM_TRY(ensure(c->tiles, tile_capacity(c, (size_t)n, tile)));
     const BucketBufs b = bucket_of(c);
     ROAM_CUDA(cudaMemsetAsync(c->aux, 0, sizeof(Counters), s));
-    launch_bucket(nullptr, nullptr, nullptr, (uint32_t)n, 1, 1, field, c->n_fields, 128, b, c->aux, grid_blocks(c, 2),
+    launch_bucket(nullptr, nullptr, nullptr, (uint32_t)n, 1, 1, field, c->n_fields, tile, b, c->aux, grid_blocks(c, 2),
                   s, c->cb);
     ROAM_TRY(launched("bucket"));
     SampleSrc src{};
@@ -1585,6 +1585,9 @@ roam_status roam_train_forward(roam_ctx *c, const roam_camera *cams, int n_views
     const int R = opts->n_max;
     if ((double)((n_rays + 31) & ~31LL) * R >= 4294967295.0) return fail(ROAM_ERR_ARG, "too many rays x samples");
     ROAM_TRY(ensure_rays(c, n_rays, R));
+    // (the SIMT adjoint's tiles may be smaller than the forward's)
+    ROAM_TRY(ensure(c->tiles, tile_capacity(c, (size_t)((n_rays + 31) & ~31LL) * (size_t)R,
+                                            mlp_bwd_simt_tile(c->md.width, c->md.n_hidden))));
     ROAM_CUDA(cudaMemsetAsync(c->ctr, 0, sizeof(Counters), s));
     ROAM_CUDA(cudaMemsetAsync(c->hist.p, 0, (size_t)c->n_fields * sizeof(uint32_t), s));
     ROAM_TRY(run_rounds(c, rays, n_rays, opts, rgb, nullptr, nullptr, R, R, s));
@@ -1621,13 +1624,15 @@ roam_status roam_train_backward(roam_ctx *c, const float *dl_drgb, float *grad, 
     ROAM_TRY(launched("composite_bwd"));
     ROAM_CUDA(cudaMemsetAsync(c->aux, 0, sizeof(Counters), s));
     const BucketBufs b = bucket_of(c);
+    const bool tc = o.precision == ROAM_BF16 && mlp_bwd_tc_supported(c->md.width, c->md.n_hidden) && c->ws[0].tc_ok;
+    const int tile = tc ? 128 : mlp_bwd_simt_tile(c->md.width, c->md.n_hidden);
     {
         ProfScope ps(c, P_BUCKET, s);
         if (fused_hist)
-            launch_bucket_ready(c->live1.p, c->recs.p, nullptr, (uint32_t)n, R, 1, c->n_fields, 128, b, c->aux,
+            launch_bucket_ready(c->live1.p, c->recs.p, nullptr, (uint32_t)n, R, 1, c->n_fields, tile, b, c->aux,
                                 grid_blocks(c, 4), s, c->cb);
         else
-            launch_bucket(c->live1.p, c->recs.p, nullptr, (uint32_t)n, R, 1, nullptr, c->n_fields, 128, b, c->aux,
+            launch_bucket(c->live1.p, c->recs.p, nullptr, (uint32_t)n, R, 1, nullptr, c->n_fields, tile, b, c->aux,
                           grid_blocks(c, 4), s, c->cb);
     }
     ROAM_TRY(launched("bucket"));
@@ -1641,7 +1646,6 @@ roam_status roam_train_backward(roam_ctx *c, const float *dl_drgb, float *grad, 
     src.st = state_of(c);
     src.delta = o.delta;
     src.accurate = o.precision == ROAM_F32;
-    const bool tc = o.precision == ROAM_BF16 && mlp_bwd_tc_supported(c->md.width, c->md.n_hidden) && c->ws[0].tc_ok;
     if (!tc) ROAM_TRY(refresh(c, o.precision, true, s));
     if (tc) {
         ProfScope ps(c, P_MLP_BWD_TC, s);
