@@ -83,6 +83,24 @@ __device__ __forceinline__ void make_ray64(const DevCamera &c, uint32_t pix, dou
     d.z = (double)c.R[6] * d0 + (double)c.R[7] * d1 + (double)c.R[8] * d2;
 }
 
+// A compile-time number as a lambda argument.
+template <int V>
+struct Int {
+    static constexpr int value = V;
+};
+
+// Asynchronous 16-byte copies from global to shared memory.
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Device counters of one render / training pass.
 struct Counters {
     uint32_t live_count[2];

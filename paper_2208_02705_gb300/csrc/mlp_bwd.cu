@@ -16,8 +16,8 @@
 //    layer overwrites the activations it belongs to, so no second buffer;
 //  - a thread owns 4 samples x TN outputs (forward, all 8 warps) or
 //    4 samples x 2 TN (dgrad, warps 0-3), while warps 4-7 form the same
-//    layer's wgrad (W/8 outputs x up to 6 inputs per thread, reduced over s
-//    in pairs): both have about the same work and share the FMA pipe;
+//    layer's wgrad (W/8 outputs x 4 inputs per thread, reduced over s in
+//    pairs): both have about the same work and share the FMA pipe;
 //  - the weights stream through a ring of shared-memory stages (16 rows each),
 //    copied asynchronously by warps 0-3 a few stages ahead, one barrier per
 //    stage: they are read once per tile and would not fit beside the gradient
@@ -66,11 +66,6 @@ struct TLayout {
           col(head + (int64_t)W * round4(1 + W) + round4(1 + W))
     {
     }
-};
-
-template <int V>
-struct Int {
-    static constexpr int value = V;
 };
 
 constexpr int kThreads = 256;
@@ -136,16 +131,6 @@ __device__ __forceinline__ float local_coord(float th0, float delta, float o, fl
     return __fadd_rn(__fadd_rn(qh, offset), ql);
 }
 
-__device__ __forceinline__ void cp_async16(void *dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-template <int N>
-__device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 // TN consecutive floats from shared memory
@@ -322,12 +307,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             *reinterpret_cast<float4 *>(row + j * XS + sF) = v;
         }
     };
-    // this tile's wgrad of one layer by kW warps (wi = this warp's index among
-    // them): g[n][k] += sum_s dz[n][s] x[k][s]; a lane owns outputs
-    // ln + 8 i and inputs kb + lk + 4 j, so a warp covers W x 4 TK
-    auto wgrad = [&](auto KK, auto KW, int wi, const float *dz, const float *x, float *g, int ldg) {
-        constexpr int K = decltype(KK)::value, TNW = W / 8;
-        constexpr int TK = (K + 4 * decltype(KW)::value - 1) / (4 * decltype(KW)::value);
+    // wgrad of K inputs of a layer by 4 warps (wi = this warp's index among
+    // them) over samples [s0, s0 + NS): g[n][k] += sum_s dz[n][s] x[k][s]; a
+    // lane owns outputs ln + 8 i and inputs kb + lk + 4 j, a warp W x 4 TK.
+    // (at most W inputs at a time: every float4 loaded from shared memory costs
+    // the FMA pipe ~5 cycles, so small TK is slow, and past TK = 4 the
+    // accumulators spill; `last` adds after the other half of the block)
+    auto wgrad = [&](auto KK, auto NSc, int wi, const float *dz, const float *x, float *g, int ldg, int s0, bool last) {
+        constexpr int K = decltype(KK)::value, TNW = W / 8, TK = (K + 15) / 16, NS = decltype(NSc)::value;
         const int ln = lane & 7, lk = lane >> 3, kb = wi * 4 * TK + lk;
         float2 acc[TNW][TK];
 #pragma unroll
@@ -339,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int j = 0; j < TK; ++j) xr[j] = x + min(kb + 4 * j, K - 1) * XS;    // (rows past K: computed, not kept)
 #pragma unroll 2
-        for (int s = 0; s < S; s += 4) {
+        for (int s = s0; s < s0 + NS; s += 4) {
             float4 xv[TK];
 #pragma unroll
             for (int j = 0; j < TK; ++j) xv[j] = *reinterpret_cast<const float4 *>(xr[j] + s);
@@ -353,6 +340,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
         }
+        if (last) sync();
 #pragma unroll
         for (int j = 0; j < TK; ++j) {
             const int k = kb + 4 * j;
@@ -584,7 +572,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
         // ---- colour, head and hidden layers: dgrad by warps 0-3 beside
         // wgrad by warps 4-7; then dX, masked, over the layer's input ----
-        auto backward = [&](auto KK, int layer, const float *dz, float *x, float *g, int ldg, int kind) {
+        auto backward = [&](int layer, const float *dz, float *x, float *g, int ldg, int kind) {
             float2 acc[4][F::TD / 2];
             if (warp < 4) {
                 // the head's density row first (kind 1), as the layer's output 0
@@ -604,9 +592,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 dense(Int<W>{}, Int<W>{}, Int<F::TD>{}, Int<128>{}, dz, kD, acc);
                 row_sums(tid, dz, nullptr, gacc + F::gB + layer * W);
+                // the colour layer's F(d) inputs beside its features' wgrad
+                if (kind == 0) wgrad(Int<kPeD>{}, Int<S>{}, warp, dz, x + W * XS, g + W, ldg, 0, false);
                 if (kind == 1) row_sums(tid, x, dzo + 3 * S, gacc + F::gDen);
             } else {
-                wgrad(KK, Int<4>{}, warp - 4, dz, x, g, ldg);
+                wgrad(Int<W>{}, Int<S>{}, warp - 4, dz, x, g, ldg, 0, false);
                 slot = (slot + W / kRingRows) % NST;
             }
             sync();
@@ -629,14 +619,16 @@ __global__ void __launch_bounds__(kThreads, 1)
             sync();
         };
         // (kind 0: the features carry no activation)
-        backward(Int<KC>{}, H + 1, X + F::rG * XS, X + F::rC * XS, gacc + F::gCol, F::SC, 0);
-        backward(Int<W>{}, H, X + F::rC * XS, X + F::rH(H) * XS, gacc + F::gHead, F::SH, 1);
+        backward(H + 1, X + F::rG * XS, X + F::rC * XS, gacc + F::gCol, F::SC, 0);
+        backward(H, X + F::rC * XS, X + F::rH(H) * XS, gacc + F::gHead, F::SH, 1);
 #pragma unroll 1
         for (int l = H - 1; l >= 1; --l)
-            backward(Int<W>{}, l, X + F::rH(l + 1) * XS, X + F::rH(l) * XS,
+            backward(l, X + F::rH(l + 1) * XS, X + F::rH(l) * XS,
                             gacc + F::gHid + (l - 1) * W * F::SH, F::SH, 2);
-        // ---- layer 1: wgrad only, by every warp ----
-        wgrad(Int<kPeX>{}, Int<8>{}, warp, X + F::rH(1) * XS, X + F::rX * XS, gacc + F::gA, F::SA);
+        // ---- layer 1: wgrad only, half of the samples by each half of the block ----
+        wgrad(Int<kPeX>{}, Int<S / 2>{}, warp & 3, X + F::rH(1) * XS, X + F::rX * XS, gacc + F::gA, F::SA,
+              warp < 4 ? 0 : S / 2, warp >= 4);
+        if (warp < 4) sync();
         if (warp < 4) row_sums(tid, X + F::rH(1) * XS, nullptr, gacc + F::gB);
     }
     sync();
