@@ -233,6 +233,7 @@ struct TeacherAffine {
 };
 int64_t teacher_param_count();
 int64_t teacher_image_bytes();
+int64_t teacher_simt_floats();       // the transposed FP32 layers
 // the caller's layout -> the tensor-core image and the transposed FP32 layers
 void launch_teacher_pack(const float *w, uint8_t *img, float *wt, cudaStream_t s);
 void launch_teacher_tc(const uint8_t *img, TeacherAffine aff, int64_t n, const float *p, const float *d, float4 *out,

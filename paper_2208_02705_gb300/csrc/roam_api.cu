@@ -1239,7 +1239,7 @@ roam_status roam_teacher_load(roam_ctx *c, const float *weights, const float *af
     // the caller's layout lands in the workspace, is checked, then packed
     // into the tensor-core image and the transposed FP32 layers
     ROAM_TRY(ensure(c->teacher_ws, (size_t)P));
-    ROAM_TRY(ensure(c->teacher_wt, (size_t)P));
+    ROAM_TRY(ensure(c->teacher_wt, (size_t)teacher_simt_floats()));
     ROAM_TRY(ensure(c->teacher_img, (size_t)teacher_image_bytes()));
     ROAM_CUDA(cudaMemcpy(c->teacher_ws.p, weights, (size_t)P * sizeof(float),
                          on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice));

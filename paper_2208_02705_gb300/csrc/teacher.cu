@@ -33,9 +33,7 @@
 // otherwise wait for a layer's MMAs: the next tile's F(x) before layer 7's
 // results (layer 5 has read the current one), its F(d) before layer 10's.
 //
-// k_teacher_simt (FP32): a plain SIMT evaluation for reference precision:
-// a block of 256 threads takes 32 points, one output unit per thread, inputs
-// in shared memory, weights read transposed ([K][N]) from global memory.
+// k_teacher_simt (FP32): a register-tiled SIMT evaluation in full precision.
 #include "tc_common.cuh"
 
 namespace roam {
@@ -474,9 +472,32 @@ __global__ void __launch_bounds__(kTThreads, 1)
 }
 
 // ---- the FP32 SIMT form ----------------------------------------------------
+//
+// Bound by the FP32 FMA pipe (1.19 MFLOP per point).  A block of 256 threads
+// takes a tile of 8 TS points: the layer's input sits in shared memory
+// feature-major (rows of 8 TS points, padded by 4), a thread owns TS points x
+// 8 outputs as packed FMAs, and the weights ([K][N]) come through a ring of
+// 16-row stages in shared memory, copied asynchronously two stages ahead (L2
+// holds them).  Every float4 read from shared memory costs the FMA pipe about
+// 5 cycles (its register writes), so TS = 16 (6 loads per 64 packed FMAs) is
+// the fastest per point; smaller tiles are for few points, where the chip
+// would be left idle (see launch_teacher_simt).  A layer's outputs replace its
+// input in place; F(x) stays in rows 256 .. 318 until layer 5 has read it, then
+// F(d) takes its place for layer 10.
+// Measured on GB300: 32,768 points 838 us (one output per thread over 32 points
+// with scalar loads of the inputs took 1955), 100,000 points 2.49 ms (5.46).
 
-constexpr int kSP = 32;          // points per block
-constexpr int kSLd = 320;        // shared activation row: [layer input (<= 256) | F(x) (63) | 0]
+constexpr int kSRows = 16;                   // weight rows per ring stage
+constexpr int kSStages = 3;
+constexpr int kSStage = kSRows * kTW;        // floats of one stage
+
+// offset of layer a in the transposed copy (every layer on a 16-byte boundary)
+__host__ __device__ constexpr int64_t ts_off(int a)
+{
+    int64_t o = 0;
+    for (int i = 0; i < a; ++i) o += ((int64_t)t_out(i) * t_in(i) + t_out(i) + 3) / 4 * 4;
+    return o;
+}
 
 // API layout -> every layer transposed ([K][N]) then its bias [N]
 __global__ void k_teacher_pack_simt(const float *__restrict__ w, float *__restrict__ wt)
@@ -484,7 +505,7 @@ __global__ void k_teacher_pack_simt(const float *__restrict__ w, float *__restri
     for (int a = 0; a < kTLayers; ++a) {
         const int N = t_out(a), K = t_in(a);
         const float *src = w + t_off(a);
-        float *dst = wt + t_off(a);
+        float *dst = wt + ts_off(a);
         for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)N * K + N;
              e += (int64_t)gridDim.x * blockDim.x) {
             if (e < (int64_t)N * K) {
@@ -497,109 +518,206 @@ __global__ void k_teacher_pack_simt(const float *__restrict__ w, float *__restri
     }
 }
 
-// one layer: Y[p][n] = act(b[n] + sum_k X[p][k] W[k][n]) for n < N, thread = n
-__device__ __forceinline__ void simt_layer(const float *__restrict__ wt, int a, const float (*X)[kSLd], float (*Y)[kSLd],
-                                           int relu)
+// the matrix layers of one tile in order: layers 1-8, the feature head, layer 10
+__host__ __device__ constexpr int ts_layer(int i) { return i < 8 ? i : i + 1; }      // 0-7, 9, 10
+
+template <int TS>
+struct TeacherSimt {
+    static constexpr int S = 8 * TS;         // points per tile
+    static constexpr int XS = S + 4;         // row stride
+    static constexpr int kX = (kTW + kPeX) * XS;
+    static constexpr size_t kSmem = (size_t)(kX + kSStages * kSStage + 256) * sizeof(float);
+};
+
+template <int TS>
+__global__ void __launch_bounds__(256, 1) k_teacher_simt(const float *__restrict__ wt, TeacherAffine aff, int64_t n,
+                                                         const float *__restrict__ p, const float *__restrict__ d,
+                                                         float4 *__restrict__ out)
 {
-    const int N = t_out(a), K = t_in(a);
-    const float *Wt = wt + t_off(a);
-    const int nn = threadIdx.x;
-    if (nn < N) {
-        float acc[kSP];
-        const float b = Wt[(int64_t)N * K + nn];
-#pragma unroll
-        for (int q = 0; q < kSP; ++q) acc[q] = b;
-        for (int k = 0; k < K; ++k) {
-            const float wk = __ldg(Wt + (int64_t)k * N + nn);
-#pragma unroll
-            for (int q = 0; q < kSP; ++q) acc[q] = fmaf(X[q][k], wk, acc[q]);
-        }
-#pragma unroll
-        for (int q = 0; q < kSP; ++q) Y[q][nn] = relu ? fmaxf(acc[q], 0.f) : acc[q];
+    using T = TeacherSimt<TS>;
+    constexpr int S = T::S, XS = T::XS, NP = 256 / S;      // NP threads per point
+    extern __shared__ float4 sm4[];
+    float *X = reinterpret_cast<float *>(sm4);             // [319][XS]
+    float *ring = X + T::kX;
+    float *red = ring + kSStages * kSStage;                // [256] partial sums
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int sg = lane & 7, og = lane >> 3;
+    const int smp = tid % S, part = tid / S;
+    __shared__ int4 lay[10];                               // offset, inputs, outputs, bias offset
+    if (tid < 10) {
+        const int a = ts_layer(tid), o = (int)ts_off(a), K = t_in(a), N = t_out(a);
+        lay[tid] = make_int4(o, K, N, o + K * N);
     }
     __syncthreads();
+
+    // the ring: stage j of the run into slot j mod kSStages; a layer's rows in order
+    int64_t issue_tile = blockIdx.x;
+    int issue_l = 0, issue_r = 0, issue_slot = 0, slot = 0;
+    const int64_t n_tiles = (n + S - 1) / S;
+    auto feed = [&]() {
+        if (issue_tile < n_tiles) {
+            const int4 L = lay[issue_l];
+            const int n4 = min(kSRows, L.y - issue_r) * L.z / 4;
+            const float *src = wt + L.x + issue_r * L.z;
+            float *dst = ring + issue_slot * kSStage;
+            for (int c = tid; c < n4; c += 256) cp_async16(dst + 4 * c, src + 4 * c);
+            if (++issue_slot == kSStages) issue_slot = 0;
+            issue_r += kSRows;
+            if (issue_r >= L.y) {
+                issue_r = 0;
+                if (++issue_l == 10) {
+                    issue_l = 0;
+                    issue_tile += gridDim.x;
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int j = 0; j + 1 < kSStages; ++j) feed();
+
+    // one layer: rows [base, base + K) of X -> rows [0, N); a warp covers 32
+    // outputs and every point (N = 128: half of the points)
+    auto layer = [&](int i, int base, bool relu) {
+        const int4 L = lay[i];
+        const int K = L.y;
+        const bool half = L.z == kTC;
+        // point groups of 4: sg + 8 g, g in [g0, g0 + ng)
+        constexpr int G = TS / 4;
+        const int col = (half ? (warp & 3) : warp) * 32 + og * 8;
+        float2 acc[TS][4];
+        {
+            const float4 *bp = reinterpret_cast<const float4 *>(wt + L.w + col);
+            const float4 b0 = __ldg(bp), b1 = __ldg(bp + 1);
+#pragma unroll
+            for (int q = 0; q < TS; ++q) {
+                acc[q][0] = make_float2(b0.x, b0.y);
+                acc[q][1] = make_float2(b0.z, b0.w);
+                acc[q][2] = make_float2(b1.x, b1.y);
+                acc[q][3] = make_float2(b1.z, b1.w);
+            }
+        }
+        auto rows = [&](auto HALF, int r0, int nr) {
+            constexpr bool kHalf = decltype(HALF)::value != 0;
+            constexpr int ng = kHalf ? (G > 1 ? G / 2 : 1) : G;
+            const int g0 = kHalf && G > 1 ? (warp >> 2) * ng : 0;
+            const float *wr = ring + slot * kSStage + col;
+            const float *xr = X + (int64_t)(base + r0) * XS + 4 * (sg + 8 * g0);
+#pragma unroll 4
+            for (int k = 0; k < nr; ++k) {
+                const float4 w0 = *reinterpret_cast<const float4 *>(wr + k * (kHalf ? kTC : kTW));
+                const float4 w1 = *reinterpret_cast<const float4 *>(wr + k * (kHalf ? kTC : kTW) + 4);
+                const float2 wv[4] = {make_float2(w0.x, w0.y), make_float2(w0.z, w0.w), make_float2(w1.x, w1.y),
+                                      make_float2(w1.z, w1.w)};
+#pragma unroll
+                for (int g = 0; g < ng; ++g) {
+                    const float4 x4 = *reinterpret_cast<const float4 *>(xr + k * XS + 32 * g);
+                    const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            acc[4 * g + q][j] = __ffma2_rn(wv[j], make_float2(xv[q], xv[q]), acc[4 * g + q][j]);
+                }
+            }
+        };
+        for (int r0 = 0; r0 < K; r0 += kSRows) {
+            // the stage has landed for every loader, and every thread is past the
+            // stage before it, whose slot takes the next copy
+            cp_async_wait<kSStages - 2>();
+            __syncthreads();
+            feed();
+            const int nr = min(kSRows, K - r0);
+            if (!half) rows(Int<0>{}, r0, nr);
+            else if (G > 1 || warp < 4) rows(Int<1>{}, r0, nr);
+            if (++slot == kSStages) slot = 0;
+        }
+        __syncthreads();                                   // every thread has read the input
+        const int ng = half ? (G > 1 ? G / 2 : (warp < 4 ? 1 : 0)) : G;
+        const int g0 = half && G > 1 ? (warp >> 2) * ng : 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                if (g >= ng) continue;
+                float v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    v[q] = (j & 1) ? acc[4 * g + q][j / 2].y : acc[4 * g + q][j / 2].x;
+                    if (relu) v[q] = fmaxf(v[q], 0.f);
+                }
+                *reinterpret_cast<float4 *>(X + (int64_t)(col + j) * XS + 4 * (sg + 8 * (g0 + g))) =
+                    make_float4(v[0], v[1], v[2], v[3]);
+            }
+        __syncthreads();
+    };
+    // F(v) of L frequencies as rows 256 .., the point's frequencies split over its threads
+    auto encode = [&](const float (&x)[3], int L) {
+        float *col = X + (int64_t)kTW * XS + smp;
+        if (part == 0)
+            for (int a = 0; a < 3; ++a) col[a * XS] = x[a];
+        for (int k = part; k < L; k += NP)
+            for (int a = 0; a < 3; ++a) {
+                float s, c;
+                sincospif(x[a] * (float)(1 << k), &s, &c);
+                col[(3 + 6 * k + a) * XS] = s;
+                col[(6 + 6 * k + a) * XS] = c;
+            }
+    };
+
+    for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+        const int64_t pt = t * S + smp;
+        float x[3];
+        load_x(p, aff, pt, n, x);
+        __syncthreads();                                   // the previous tile's last reads
+        encode(x, 10);
+        __syncthreads();
+        layer(0, kTW, true);
+#pragma unroll 1
+        for (int i = 1; i < 5; ++i) layer(i, 0, true);     // layer 5 on [h4 | F(x)]
+        // F(x) has been read: F(d) takes its rows (read by layer 10, syncs in between)
+        load_d(d, pt, n, x);
+        encode(x, 4);
+#pragma unroll 1
+        for (int i = 5; i < 8; ++i) layer(i, 0, i < 7);    // layer 8 is linear
+        // density head: a point's threads split the sum
+        {
+            const float *Wd = wt + ts_off(8);
+            float s = 0.f;
+#pragma unroll 8
+            for (int k = part * (kTW / NP); k < (part + 1) * (kTW / NP); ++k) s = fmaf(X[(int64_t)k * XS + smp], __ldg(Wd + k), s);
+            red[tid] = s;
+        }
+        __syncthreads();
+        float sigma = 0.f;
+        if (part == 0) {
+            for (int q = 0; q < NP; ++q) sigma += red[q * S + smp];
+            sigma = fmaxf(sigma + __ldg(wt + ts_off(8) + kTW), 0.f);
+        }
+        layer(8, 0, true);                                 // feature head
+        layer(9, 0, true);                                 // layer 10 on [feature | F(d)]
+        if (part == 0 && pt < n) {
+            const float *Wo = wt + ts_off(11);             // [128][3] then bias[3]
+            float z[3] = {__ldg(Wo + 3 * kTC), __ldg(Wo + 3 * kTC + 1), __ldg(Wo + 3 * kTC + 2)};
+#pragma unroll 8
+            for (int k = 0; k < kTC; ++k) {
+                const float g = X[(int64_t)k * XS + smp];
+                for (int c = 0; c < 3; ++c) z[c] = fmaf(g, __ldg(Wo + 3 * k + c), z[c]);
+            }
+            out[pt] = make_float4(sigma, 1.f / (1.f + expf(-z[0])), 1.f / (1.f + expf(-z[1])), 1.f / (1.f + expf(-z[2])));
+        }
+    }
 }
 
-__global__ void __launch_bounds__(256) k_teacher_simt(const float *__restrict__ wt, TeacherAffine aff, int64_t n,
-                                                      const float *__restrict__ p, const float *__restrict__ d,
-                                                      float4 *__restrict__ out)
+template <int TS>
+void launch_simt_t(const float *wt, TeacherAffine aff, int64_t n, const float *p, const float *d, float4 *out, int n_sm,
+                   cudaStream_t s)
 {
-    extern __shared__ float sm[];
-    float(*X)[kSLd] = reinterpret_cast<float(*)[kSLd]>(sm);
-    float(*Y)[kSLd] = reinterpret_cast<float(*)[kSLd]>(sm + kSP * kSLd);
-    __shared__ float fd[kSP][kPeD];
-    __shared__ float sig[kSP];
-    for (int64_t base = (int64_t)blockIdx.x * kSP; base < n; base += (int64_t)gridDim.x * kSP) {
-        // encodings: F(x) at columns 0..62 of X (layer 1's input) and again at
-        // 256..318 of Y (the skip into layer 5); F(d) aside
-        for (int q = threadIdx.x; q < kSP; q += blockDim.x) {
-            const int64_t i = base + q;
-            float x[3] = {0.f, 0.f, 0.f}, dv[3] = {0.f, 0.f, 1.f};
-            if (i < n)
-                for (int a = 0; a < 3; ++a) {
-                    x[a] = fmaf(aff.v[a], p[3 * i + a], aff.v[3 + a]);
-                    dv[a] = d[3 * i + a];
-                }
-            for (int a = 0; a < 3; ++a) {
-                X[q][a] = x[a];
-                fd[q][a] = dv[a];
-            }
-            for (int k = 0; k < 10; ++k)
-                for (int a = 0; a < 3; ++a) {
-                    float s, c;
-                    sincospif(x[a] * (float)(1 << k), &s, &c);
-                    X[q][3 + 6 * k + a] = s;
-                    X[q][6 + 6 * k + a] = c;
-                }
-            for (int k = 0; k < 4; ++k)
-                for (int a = 0; a < 3; ++a) {
-                    float s, c;
-                    sincospif(dv[a] * (float)(1 << k), &s, &c);
-                    fd[q][3 + 6 * k + a] = s;
-                    fd[q][6 + 6 * k + a] = c;
-                }
-            for (int k = 0; k < kPeX; ++k) Y[q][kTW + k] = X[q][k];
-        }
-        __syncthreads();
-        simt_layer(wt, 0, X, Y, 1);                  // layer 1 -> Y[0..255]; Y keeps F(x) at 256..318
-        simt_layer(wt, 1, Y, X, 1);
-        simt_layer(wt, 2, X, Y, 1);
-        // layer 4 writes X; layer 5 reads [X | F(x)]: copy F(x) beside it
-        for (int e = threadIdx.x; e < kSP * kPeX; e += blockDim.x) X[e / kPeX][kTW + e % kPeX] = Y[e / kPeX][kTW + e % kPeX];
-        simt_layer(wt, 3, Y, X, 1);
-        simt_layer(wt, 4, X, Y, 1);                  // layer 5 on [h4 | F(x)]
-        simt_layer(wt, 5, Y, X, 1);
-        simt_layer(wt, 6, X, Y, 1);
-        simt_layer(wt, 7, Y, X, 0);                  // layer 8, linear
-        // density head: one warp per point group
-        {
-            const float *Wd = wt + t_off(8);
-            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-            for (int q = warp; q < kSP; q += blockDim.x >> 5) {
-                float s = 0.f;
-                for (int k = lane; k < kTW; k += 32) s = fmaf(X[q][k], Wd[k], s);
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) sig[q] = fmaxf(s + Wd[kTW], 0.f);
-            }
-        }
-        simt_layer(wt, 9, X, Y, 1);                  // feature head -> Y[0..255]
-        for (int e = threadIdx.x; e < kSP * kPeD; e += blockDim.x) Y[e / kPeD][kTW + e % kPeD] = fd[e / kPeD][e % kPeD];
-        __syncthreads();
-        simt_layer(wt, 10, Y, X, 1);                 // layer 10 on [feature | F(d)] -> X[0..127]
-        {
-            const float *Wo = wt + t_off(11);         // [128][3] then bias[3]
-            for (int q = threadIdx.x; q < kSP; q += blockDim.x) {
-                float z[3] = {Wo[3 * kTC], Wo[3 * kTC + 1], Wo[3 * kTC + 2]};
-                for (int k = 0; k < kTC; ++k)
-                    for (int c = 0; c < 3; ++c) z[c] = fmaf(X[q][k], Wo[3 * k + c], z[c]);
-                const int64_t i = base + q;
-                if (i < n)
-                    out[i] = make_float4(sig[q], 1.f / (1.f + expf(-z[0])), 1.f / (1.f + expf(-z[1])),
-                                         1.f / (1.f + expf(-z[2])));
-            }
-        }
-        __syncthreads();
-    }
+    using T = TeacherSimt<TS>;
+    static int smem_set[kMaxDevices] = {};
+    raise_smem_limit((const void *)k_teacher_simt<TS>, (int)T::kSmem, smem_set);
+    const int64_t tiles = (n + T::S - 1) / T::S;
+    k_teacher_simt<TS><<<(int)(tiles < n_sm ? tiles : n_sm), 256, T::kSmem, s>>>(wt, aff, n, p, d, out);
 }
 
 }  // namespace
@@ -625,15 +743,19 @@ void launch_teacher_tc(const uint8_t *img, TeacherAffine aff, int64_t n, const f
     if (grid > 0) k_teacher_tc<<<grid, kTThreads, smem, s>>>(img, aff, n, p, d, out, status);
 }
 
+int64_t teacher_simt_floats() { return ts_off(kTLayers); }
+
 void launch_teacher_simt(const float *wt, TeacherAffine aff, int64_t n, const float *p, const float *d, float4 *out,
                          int n_sm, cudaStream_t s)
 {
-    const int smem = 2 * kSP * kSLd * (int)sizeof(float);
-    static int smem_set[kMaxDevices] = {};
-    raise_smem_limit((const void *)k_teacher_simt, smem, smem_set);
-    const int64_t blocks = (n + kSP - 1) / kSP;
-    const int grid = (int)(blocks < 4 * n_sm ? blocks : 4 * n_sm);
-    if (grid > 0) k_teacher_simt<<<grid, 256, smem, s>>>(wt, aff, n, p, d, out);
+    if (n <= 0) return;
+    // one tile per block at a time: the tile size whose waves end first, from
+    // the measured time of one tile of 128 / 64 / 32 points (424 / 248 / 164 us)
+    auto waves = [&](int S) { return (double)(((n + S - 1) / S + n_sm - 1) / n_sm); };
+    const double c16 = 424 * waves(128), c8 = 248 * waves(64), c4 = 164 * waves(32);
+    if (c16 <= c8 && c16 <= c4) launch_simt_t<16>(wt, aff, n, p, d, out, n_sm, s);
+    else if (c8 <= c4) launch_simt_t<8>(wt, aff, n, p, d, out, n_sm, s);
+    else launch_simt_t<4>(wt, aff, n, p, d, out, n_sm, s);
 }
 
 }  // namespace roam
