@@ -242,9 +242,9 @@ void launch_teacher_simt(const float *wt, TeacherAffine aff, int64_t n, const fl
                          int n_sm, cudaStream_t s);
 void launch_distill_loss(int64_t n, const float4 *student, const float4 *teacher, float I, float4 *dl, float *loss,
                          cudaStream_t s);
-size_t assign_scratch_bytes();
-void launch_assign(const uint32_t *bits, const uint32_t *prefix, int64_t n_words, int gx, int gy, uint32_t S, int n,
-                   uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm, cudaStream_t s);
+size_t assign_scratch_bytes(uint32_t S, int64_t n_bricks);
+void launch_assign(const uint32_t *bits, const uint32_t *prefix, int64_t n_words, int gx, int gy, int gz, uint32_t S,
+                   int n, uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm, cudaStream_t s);
 uint32_t assign_status(const void *scratch);
 void launch_occupancy_scan(const GridDev &g, const DevCamera *cams, int view, int n_pix, const float *depth,
                            const float *opacity, const roam_occ_params &q, uint32_t *hit, uint32_t *free_bits,

@@ -1221,8 +1221,8 @@ roam_status roam_assign_fields(roam_ctx *c, int n_fields, uint16_t *labels, int3
     if (S >= (int64_t)1 << 27) return fail(ROAM_ERR_ARG, "at most 2^27 - 1 occupied voxels");
     cudaStream_t s = (cudaStream_t)stream;
     ROAM_TRY(ensure(c->assign_vox, (size_t)S));
-    ROAM_TRY(ensure(c->assign_scratch, assign_scratch_bytes()));
-    launch_assign(c->bits.p, c->prefix.p, c->n_words, c->g.gx, c->g.gy, (uint32_t)S, n_fields, c->assign_vox.p,
+    ROAM_TRY(ensure(c->assign_scratch, assign_scratch_bytes((uint32_t)S, (int64_t)c->g.bx * c->g.by * c->g.bz)));
+    launch_assign(c->bits.p, c->prefix.p, c->n_words, c->g.gx, c->g.gy, c->g.gz, (uint32_t)S, n_fields, c->assign_vox.p,
                   labels, boxes, c->assign_scratch.p, c->n_sm, s);
     ROAM_TRY(launched("field assignment"));
     ROAM_CUDA(cudaStreamSynchronize(s));
