@@ -61,21 +61,24 @@ __device__ __forceinline__ void st_words32(uint32_t tArow, int c, const uint32_t
 }
 
 // Persistent kernel, one CTA per SM, kSlots tiles in flight.  Slot s is
-// warpgroup s: its 128 threads encode and run the epilogues of their tile
-// (one row each), and its first thread issues the tile's MMAs itself --
+// warpgroup s (W = 128: warpgroups 2 s and 2 s + 1, each with half of every
+// row's columns): its threads encode and run the epilogues of their tile
+// (one row each), and one of them issues the tile's MMAs itself --
 // tcgen05.mma and tcgen05.commit occupy the issuing thread for tens to
 // hundreds of cycles each, so one issuer per slot lets the slots' chains
 // overlap.  Tiles come in field-uniform groups of kSlots (bucket padding);
 // at a field change all slots meet at a CTA barrier, thread 0 reloads the
 // shared weight image, and each issuer waits for it before its next MMA.
 template <int W, int H, bool F8>
-__global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
+__global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * TcShape<W, H, F8>::kSlotThreads, 1)
     k_mlp_tc(const void *wimg, int64_t img_bytes, int field_base, int cls, const float *affine, float sig_scale,
              int act, SampleSrc src, BucketBufs b, Counters *ctr, float4 *out, unsigned long long wait_ns,
              int withhold_image)
 {
     using S = TcShape<W, H, F8>;
     constexpr int kSlots = S::kSlots;
+    constexpr int CG = S::kColGroups, ST = S::kSlotThreads;
+    constexpr int NC = W / CG;                       // columns of one warpgroup's share of a row
     constexpr int kLayers = S::kLayers;
     constexpr int kStageRec = kLayers >= 4 ? 1 : 0;  // the layer after which the next tile's records are gathered
     constexpr int kCols = S::kSlotCols;
@@ -87,15 +90,17 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
     __shared__ uint64_t bar_w;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ float4 part[CG > 1 ? kSlots * 128 : 1];       // the second warpgroup's share of the 3 outputs
 
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *IMG = smem_raw + (base - smem_u32(smem_raw));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int slot = warp >> 2, wq = warp & 3;
+    const int slot = warp / (4 * CG), cg = CG > 1 ? (warp >> 2) % CG : 0, wq = warp & 3;
+    const int c0 = cg * NC;                                   // this thread's first column
     const int row = wq * 32 + lane;                           // TMEM lane == tile row
     // the slot's issuing thread sits in the slot's warp with index = slot mod 4,
     // so the slots' issuers run on different SM sub-partitions
-    const bool issuer = wq == (slot & 3) && lane == 0;
+    const bool issuer = wq == (slot & 3) && lane == 0 && cg == 0;
     volatile int *abortp = &abort_flag;
     uint32_t *status = &ctr->status;
 
@@ -128,6 +133,10 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
     const uint32_t g0 = (uint32_t)((uint64_t)n_groups * blockIdx.x / gridDim.x);
     const uint32_t g1 = (uint32_t)((uint64_t)n_groups * (blockIdx.x + 1) / gridDim.x);
 
+    // the two warps of the same 32 rows (two warpgroups per slot)
+    auto row_sync = [&]() {
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + kSlots + slot * 4 + wq), "r"(64) : "memory");
+    };
     uint32_t d_ph = 0, n_changes = 0, n_commits = 0, n_waits = 0;
     uint32_t cur_field = 0xffffffffu;
     bool w_ready = false, w_waited_last = true;
@@ -158,7 +167,7 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
             fence_async_smem();
             // every slot has waited on its last layer, so no MMA reads the old
             // image; meet (and agree on any abort), reload, issuers wait below
-            if (named_sync_or(15, kSlots * 128, aborted || *abortp)) break;
+            if (named_sync_or(15, kSlots * ST, aborted || *abortp)) break;
             if (threadIdx.x == 0 && !withhold_image) {
                 // each phase of bar_w carries exactly one arrival and one image
                 mbar_expect_tx(&bar_w, (uint32_t)S::kImageBytes);
@@ -179,14 +188,14 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
         const Tile cur = tl;
         const SampleIn sm = nxt;
         if (g + 1 < g1) tl = tiles[(g + 1) * kSlots + slot];
-        if (cur.count == 0 || aborted) {
+        if (cur.count == 0) {
             if (g + 1 < g1) nxt = fetch_sample(src, b, tl, row);
             continue;
         }
         const bool valid = (uint32_t)row < cur.count;
         const float *aff = affine + 6 * (int64_t)cur.field;
-        // ---- L1 input: [F(x_loc) | 1] ----
-        {
+        // ---- L1 input: [F(x_loc) | 1] (with two warpgroups, by the first) ----
+        if (cg == 0) {
             const float xl[3] = {fmaf(__ldg(aff + 0), sm.px, __ldg(aff + 3)), fmaf(__ldg(aff + 1), sm.py, __ldg(aff + 4)),
                                  fmaf(__ldg(aff + 2), sm.pz, __ldg(aff + 5))};
             // rows past the tile's count compute garbage that is never stored
@@ -200,10 +209,10 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
         float sigma = 0.f;
 #pragma unroll 1
         for (int l = 0; l < kLayers; ++l) {
-            // A for layer l is complete once all 128 threads of the slot arrive
+            // A for layer l is complete once all threads of the slot arrive
             tmem_wait_st();
             tc_fence_before();
-            if (named_sync_or(1 + slot, 128, aborted || *abortp)) {
+            if (named_sync_or(1 + slot, ST, aborted || *abortp)) {
                 aborted = true;
                 break;
             }
@@ -235,7 +244,8 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
                 encode_packed<F8, 4, 1, false, 32>(dv, w);
                 st_words32<F8>(tArow, W / 32, w);
             };
-            if (W >= 64 && l == 0) store_tail();
+            // (with two warpgroups by the second, which has no encoding of its own)
+            if (W >= 64 && l == 0 && cg == CG - 1) store_tail();
             const bool got = mbar_wait(&bar_d[slot], d_ph, abortp, status, false, wait_ns);
             if (issuer && got) ++n_waits;
             d_ph ^= 1u;
@@ -243,6 +253,8 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
             // slot decides together at the next barrier
             if (!__all_sync(0xffffffffu, got)) {
                 aborted = true;
+                // (the other warp of these rows may have gone on to their meeting)
+                if (CG > 1 && l == H + 1) row_sync();
                 continue;
             }
             tc_fence_after();
@@ -273,7 +285,7 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
                 // next activations, 32 columns at a time (few live registers):
                 // head features stay linear, every other layer ReLU
 #pragma unroll
-                for (int c = 0; c < W / 32; ++c) {
+                for (int c = c0 / 32; c < c0 / 32 + NC / 32; ++c) {
                     uint32_t r32[32];
                     tmem_ld32_nowait(trow + 32 * c, r32);
                     tmem_wait_ld();
@@ -304,7 +316,7 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
                 }
                 }
                 if (W < 64 && l == 0) store_tail();
-                if (l == H) {
+                if (l == H && cg == 0) {
                     // density from column W of the head
                     float sl = __uint_as_float(tmem_ld1(trow + W));
                     tmem_wait_ld();
@@ -322,13 +334,14 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
                 float2 ax = make_float2(0.f, 0.f), ay = ax, az = ax;
                 // chunk c + 1's TMEM load in flight during chunk c's FMAs
                 uint32_t ra[16], rb[16];
-                tmem_ld16_nowait(trow, ra);
+                tmem_ld16_nowait(trow + c0, ra);
                 tmem_wait_ld();
 #pragma unroll
-                for (int c = 0; c < W / 16; ++c) {
-                    uint32_t(&r)[16] = (c & 1) ? rb : ra;
-                    uint32_t(&nxt)[16] = (c & 1) ? ra : rb;
-                    if (c + 1 < W / 16) tmem_ld16_nowait(trow + 16 * (c + 1), nxt);
+                for (int cc = 0; cc < NC / 16; ++cc) {
+                    const int c = c0 / 16 + cc;
+                    uint32_t(&r)[16] = (cc & 1) ? rb : ra;
+                    uint32_t(&nxt)[16] = (cc & 1) ? ra : rb;
+                    if (cc + 1 < NC / 16) tmem_ld16_nowait(trow + 16 * (c + 1), nxt);
                     float gk[16];
                     if constexpr (F8) {
                         // y = s z + b per channel, packed pairs (each half rounded as fmaf)
@@ -362,11 +375,24 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * 128, 1)
                         az = __ffma2_rn(make_float2(wz.x, wz.y), g01, az);
                         az = __ffma2_rn(make_float2(wz.z, wz.w), g23, az);
                     }
-                    if (c + 1 < W / 16) tmem_wait_ld();
+                    if (cc + 1 < NC / 16) tmem_wait_ld();
                 }
                 const float4 bo = *reinterpret_cast<const float4 *>(wo + 4 * W);
-                const float4 acc = make_float4(bo.x + (ax.x + ax.y), bo.y + (ay.x + ay.y), bo.z + (az.x + az.y), 0.f);
-                if (valid) out[sm.idx] = make_float4(sigma, sigmoid_f(acc.x), sigmoid_f(acc.y), sigmoid_f(acc.z));
+                float4 acc = make_float4(ax.x + ax.y, ay.x + ay.y, az.x + az.y, 0.f);
+                if constexpr (CG > 1) {
+                    // the two warps of a row meet; the next tile's shares come
+                    // after the slot's barriers in between
+                    if (cg == 1) part[slot * 128 + row] = acc;
+                    row_sync();
+                    if (cg == 0) {
+                        const float4 q = part[slot * 128 + row];
+                        acc.x += q.x;
+                        acc.y += q.y;
+                        acc.z += q.z;
+                    }
+                }
+                acc = make_float4(bo.x + acc.x, bo.y + acc.y, bo.z + acc.z, 0.f);
+                if (valid && cg == 0) out[sm.idx] = make_float4(sigma, sigmoid_f(acc.x), sigmoid_f(acc.y), sigmoid_f(acc.z));
             }
             tc_fence_before();
             // each gather stage a layer or more after the load it depends on
@@ -636,7 +662,7 @@ void launch_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Co
     raise_smem_limit((const void *)k_mlp_tc<W, H, F8>, smem, smem_set);
     const void *img = F8 ? w.wimg8 : w.wimg;
     const int64_t ib = F8 ? w.img8_bytes : w.img_bytes;
-    k_mlp_tc<W, H, F8><<<n_sm, kSlots * 128, smem, s>>>(img, ib, w.field_base, w.cls, w.affine, w.sigma_scale, w.act,
+    k_mlp_tc<W, H, F8><<<n_sm, kSlots * TcShape<W, H, F8>::kSlotThreads, smem, s>>>(img, ib, w.field_base, w.cls, w.affine, w.sigma_scale, w.act,
                                                         src, b, ctr, out, w.wait_ns ? w.wait_ns : kWaitNs,
                                                         w.withhold_image);
 }

@@ -53,6 +53,11 @@ struct TcShape {
     static constexpr int kACols = K_COL * kEB / 4;
     static constexpr int kSlotCols = kDCols + kACols;
     static constexpr int kSlots = 512 / kSlotCols >= 4 ? 4 : (512 / kSlotCols >= 2 ? 2 : 1);
+    // warpgroups per slot, each with its share of a row's columns: TMEM admits
+    // only two slots at W = 128, whose epilogues would leave most issue slots
+    // empty with one warpgroup each
+    static constexpr int kColGroups = kSlots >= 4 ? 1 : 2;
+    static constexpr int kSlotThreads = 128 * kColGroups;
 };
 
 // ---- PTX wrappers ----
@@ -257,6 +262,16 @@ __device__ __forceinline__ uint32_t pack_e4m3x4(float a, float b, float c, float
     return (uint32_t)lo | ((uint32_t)hi << 16);
 }
 
+// the same through a ReLU fused into the conversion (the inputs are never NaN:
+// s D + b with finite terms)
+__device__ __forceinline__ uint32_t pack_e4m3x4_relu(float a, float b, float c, float d)
+{
+    uint16_t lo, hi;
+    asm("cvt.rn.satfinite.relu.e4m3x2.f32 %0, %2, %1;" : "=h"(lo) : "f"(a), "f"(b));
+    asm("cvt.rn.satfinite.relu.e4m3x2.f32 %0, %2, %1;" : "=h"(hi) : "f"(c), "f"(d));
+    return (uint32_t)lo | ((uint32_t)hi << 16);
+}
+
 __device__ __forceinline__ uint32_t pack_bf16_relu(float a, float b)
 {
     uint32_t r;
@@ -272,13 +287,9 @@ __device__ __forceinline__ void st_act32(uint32_t tArow, int c, const float (&v)
     if constexpr (F8) {
         uint32_t o[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float a0 = kRelu ? fmaxf(v[4 * q], 0.f) : v[4 * q];
-            const float a1 = kRelu ? fmaxf(v[4 * q + 1], 0.f) : v[4 * q + 1];
-            const float a2 = kRelu ? fmaxf(v[4 * q + 2], 0.f) : v[4 * q + 2];
-            const float a3 = kRelu ? fmaxf(v[4 * q + 3], 0.f) : v[4 * q + 3];
-            o[q] = pack_e4m3x4(a0, a1, a2, a3);
-        }
+        for (int q = 0; q < 8; ++q)
+            o[q] = kRelu ? pack_e4m3x4_relu(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3])
+                         : pack_e4m3x4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         tmem_st8(tArow + 8 * c, o);
     } else {
         uint32_t o[16];
