@@ -246,9 +246,16 @@ size_t assign_scratch_bytes(uint32_t S, int64_t n_bricks);
 void launch_assign(const uint32_t *bits, const uint32_t *prefix, int64_t n_words, int gx, int gy, int gz, uint32_t S,
                    int n, uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm, cudaStream_t s);
 uint32_t assign_status(const void *scratch);
-void launch_occupancy_scan(const GridDev &g, const DevCamera *cams, int view, int n_pix, const float *depth,
-                           const float *opacity, const roam_occ_params &q, uint32_t *hit, uint32_t *free_bits,
-                           float *logit, uint32_t *bits, int n_sm, cudaStream_t s);
+size_t occupancy_view_bytes(int n_views);
+// per view: what its rays share (`views`), and the sines and cosines of its
+// columns and rows (`tab`: width + height entries per equirectangular view)
+void launch_occupancy_views(const GridDev &g, const DevCamera *cams, int n_views, void *views, double2 *tab,
+                            cudaStream_t s);
+// hit, free_bits and hit_bits are zero before and after; bits may be nullptr
+void launch_occupancy_scan(const GridDev &g, const DevCamera *cams, int view, int n_pix, const void *views,
+                           const double2 *tab, const float *depth, const float *opacity, const roam_occ_params &q,
+                           uint32_t *hit, uint32_t *free_bits, uint32_t *hit_bits, float *logit, uint32_t *bits, int n_sm,
+                           cudaStream_t s);
 // tiles of `tile` samples, every non-empty field's tile count rounded up to a
 // multiple of `group`; with hist_ready the histogram is already in b.hist
 void launch_bucket_ready(const uint32_t *cnt, const uint32_t *recs, const uint32_t *live_count,

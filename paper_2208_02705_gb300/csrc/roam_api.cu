@@ -142,7 +142,10 @@ struct roam_ctx {
     DBuf<Tile> tiles;
     DBuf<float> o_rgb, o_depth, o_op;
     DBuf<DevCamera> cams;
-    DBuf<uint32_t> occ_hit, occ_free;        // occupancy update marks (per voxel, per 32 voxels)
+    DBuf<uint32_t> occ_hit, occ_free;        // occupancy update marks (per voxel; 2 words per 32 voxels)
+    bool occ_clean = false;                  // the marks are zero (a scan leaves them so)
+    DBuf<uint8_t> occ_views;
+    DBuf<double2> occ_tab;
     DBuf<uint32_t> assign_vox;               // occupied voxels' linear indices (field assignment)
     // distillation teacher (global 360NeRF)
     bool has_teacher = false;
@@ -819,7 +822,7 @@ roam_status roam_destroy(roam_ctx *c)
     for (WSet &q : c->ws) {
         release(q.w32); release(q.wt); release(q.wr); release(q.wimg); release(q.wimg8);
     }
-    release(c->occ_hit); release(c->occ_free); release(c->assign_vox); release(c->assign_scratch);
+    release(c->occ_hit); release(c->occ_free); release(c->occ_views); release(c->occ_tab); release(c->assign_vox); release(c->assign_scratch);
     release(c->teacher_img); release(c->teacher_wt); release(c->teacher_ws); release(c->selftest);
     release(c->perm); release(c->inv); release(c->labels_orig); release(c->keys_tmp);
     release(c->gsr); release(c->adam_m); release(c->adam_v);
@@ -1197,15 +1200,33 @@ roam_status roam_occupancy_update(roam_ctx *c, const roam_camera *cams, int n_vi
     int64_t n_pix = 0;
     ROAM_TRY(upload_cams(c, cams, n_views, 0.25f * c->gd.vox, &n_pix, s));
     const int64_t n_vox = (int64_t)c->g.gx * c->g.gy * c->g.gz;
+    const size_t n_words = (size_t)(n_vox / 32);
+    if (c->occ_hit.n < (size_t)n_vox || c->occ_free.n < 2 * n_words) c->occ_clean = false;
     ROAM_TRY(ensure(c->occ_hit, (size_t)n_vox));
-    ROAM_TRY(ensure(c->occ_free, (size_t)(n_vox / 32)));
-    ROAM_CUDA(cudaMemsetAsync(c->occ_hit.p, 0, (size_t)n_vox * 4, s));
-    ROAM_CUDA(cudaMemsetAsync(c->occ_free.p, 0, (size_t)(n_vox / 32) * 4, s));
+    ROAM_TRY(ensure(c->occ_free, 2 * n_words));
+    ROAM_TRY(ensure(c->occ_views, occupancy_view_bytes(n_views)));
+    size_t n_tab = 0;
+    for (int v = 0; v < n_views; ++v)
+        if (cams[v].model == ROAM_EQUIRECT) n_tab += (size_t)cams[v].width + (size_t)cams[v].height;
+    ROAM_TRY(ensure(c->occ_tab, n_tab));
+    // (a captured call clears them itself: it may be replayed in any order)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    ROAM_CUDA(cudaStreamIsCapturing(s, &cap));
+    const bool capturing = cap != cudaStreamCaptureStatusNone;
+    if (!c->occ_clean || capturing) {
+        ROAM_CUDA(cudaMemsetAsync(c->occ_hit.p, 0, c->occ_hit.n * 4, s));
+        ROAM_CUDA(cudaMemsetAsync(c->occ_free.p, 0, c->occ_free.n * 4, s));
+    }
+    c->occ_clean = false;
+    launch_occupancy_views(c->g, c->cams.p, n_views, c->occ_views.p, c->occ_tab.p, s);
+    ROAM_TRY(launched("occupancy views"));
     for (int v = 0; v < n_views; ++v) {
-        launch_occupancy_scan(c->g, c->cams.p, v, cams[v].width * cams[v].height, depth, opacity, *q, c->occ_hit.p,
-                              c->occ_free.p, logit, bits, c->n_sm, s);
+        launch_occupancy_scan(c->g, c->cams.p, v, cams[v].width * cams[v].height, c->occ_views.p, c->occ_tab.p, depth,
+                              opacity, *q, c->occ_hit.p, c->occ_free.p, c->occ_free.p + n_words, logit,
+                              v + 1 == n_views ? bits : nullptr, c->n_sm, s);
         ROAM_TRY(launched("occupancy scan"));
     }
+    c->occ_clean = !capturing;
     c->last = s;
     return ROAM_OK;
 }
