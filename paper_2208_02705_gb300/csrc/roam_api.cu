@@ -420,11 +420,11 @@ roam_status upload_cams(roam_ctx *c, const roam_camera *cams, int n_views, float
 }
 
 // tile records needed for `samples` samples in tiles of `tile`: each field's
-// run rounded up to its padding (at most the larger of 8 and the forced
-// padding)
+// run rounded up to its padding (at most 8, or the forced padding rounded up
+// to a kernel's tiles in flight)
 size_t tile_capacity(const roam_ctx *c, size_t samples, int tile = 128)
 {
-    return samples / (size_t)tile + (size_t)c->n_fields * (size_t)std::max(8, c->tile_pad) + 1;
+    return samples / (size_t)tile + (size_t)c->n_fields * (size_t)(c->tile_pad + 8) + 1;
 }
 
 roam_status ensure_rays(roam_ctx *c, int64_t n_rays, int R)
@@ -490,17 +490,18 @@ BucketBufs bucket_of(roam_ctx *c)
 int tile_of(int precision) { return precision != ROAM_F32 ? tc_tile_samples() : 128; }
 // The classes with the tile padding of their MLP kernels: on the tensor cores
 // every field's tile run is a multiple of its own kernel's tiles in flight
-// (4, or 2 at W = 128), so that no group of tiles is empty throughout; the
-// classes come in increasing width and the counts do not grow with width,
-// so each class's range still starts on a group boundary of its kernel.
-// FP32 (SIMT, one tile at a time): no padding.
+// (6 / 4 / 2 at W = 32 / 64 / 128), so that no group of tiles is empty
+// throughout and a class's groups, counted from its first tile, never mix
+// fields.  FP32 (SIMT, one tile at a time): no padding.
 ClassBounds classes_of(const roam_ctx *c, int precision)
 {
     ClassBounds cb = c->cb;
-    for (int k = 0; k < 4; ++k)
-        cb.group[k] = (precision != ROAM_F32 && k < c->n_ws)
-                          ? (c->tile_pad > 0 ? c->tile_pad : tc_tile_group(c->ws[k].W, precision == ROAM_FP8))
-                          : 1;
+    for (int k = 0; k < 4; ++k) {
+        cb.group[k] = 1;
+        if (precision == ROAM_F32 || k >= c->n_ws) continue;
+        const int g = tc_tile_group(c->ws[k].W, precision == ROAM_FP8);
+        cb.group[k] = std::max(1, (c->tile_pad + g - 1) / g) * g;
+    }
     return cb;
 }
 
@@ -1380,8 +1381,7 @@ roam_status roam_get_stats(roam_ctx *c, roam_stats *st)
 roam_status roam_set_tile_padding(roam_ctx *c, int tiles)
 {
     ROAM_TRY(set_dev(c));
-    // a multiple of every tensor-core kernel's tiles in flight (4, 2 or 1),
-    // so that every width class's range still starts on a group boundary
+    // (each width class rounds it up to its own kernel's tiles in flight)
     if (tiles != 0 && (tiles < 4 || tiles > 64 || tiles % 4))
         return fail(ROAM_ERR_ARG, "tile padding must be 0 or a multiple of 4 in [4, 64]");
     c->tile_pad = tiles;
