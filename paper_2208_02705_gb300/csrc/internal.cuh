@@ -267,8 +267,16 @@ void launch_bucket(const uint32_t *cnt, const uint32_t *recs, const uint32_t *li
                    cudaStream_t s, ClassBounds cb);
 void launch_mlp_simt(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b,
                      Counters *ctr, float4 *out, int n_sm, cudaStream_t s);
-void launch_pack_simt(const float *w32, int n_fields, int W, int H, int64_t P, float *wt,
-                      int64_t Pt, cudaStream_t s);
+// The derived copies of n_fields fields' parameters at src (API layout), each
+// where its pointer is set: the masters themselves (w32), the transposed copy
+// (wt), the dgrad copy (wr), the BF16 and E4M3 images; a NaN or infinity sets *bad.
+struct PackDst {
+    float *w32, *wt, *wr;
+    uint8_t *img, *img8;
+    int64_t img_bytes, img8_bytes;
+    uint32_t *bad;
+};
+void launch_pack(const float *src, int n_fields, int W, int H, int64_t P, const PackDst &d, cudaStream_t s);
 int64_t simt_transposed_size(int W, int H);
 void launch_composite_round(const MarchParams &mp, const float4 *sr, uint32_t *next_live,
                             uint32_t *next_count, float t_stop, const float *bg, float *rgb,
@@ -289,8 +297,6 @@ int mlp_bwd_simt_tile(int W, int H);      // samples per tile of the SIMT adjoin
 bool mlp_bwd_tc_supported(int W, int H);
 void launch_mlp_bwd_tc(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr,
                        const float4 *gsr, float *grad, int n_sm, cudaStream_t s);
-void launch_pack_rows(const float *w32, int n_fields, int W, int H, int64_t P, float *wr, int64_t Pr,
-                      cudaStream_t s);
 int64_t rows_padded_size(int W, int H);
 void launch_l2_loss(int64_t n_rays, const float *rgb, const float *target, float norm, float *dl, float *loss,
                     cudaStream_t s);
@@ -305,8 +311,6 @@ bool tc_supported(int W, int H, bool f8);
 int64_t tc_image_bytes(int W, int H, bool f8);
 int tc_tile_samples();
 int tc_tile_group(int W, bool f8);
-void launch_pack_tc(const float *w32, int n_fields, int W, int H, int64_t P, void *wimg, int64_t img_bytes, bool f8,
-                    cudaStream_t s);
 // Adam fused with the BF16 image refresh (W <= 64); false: not available for this shape
 bool launch_adam_tc(float *w32, float *m, float *v, const float *g, int n_fields, int W, int H, int64_t P, void *wimg,
                     int64_t img_bytes, float lr, float b1, float b2, float eps, float bc1, float bc2, cudaStream_t s);

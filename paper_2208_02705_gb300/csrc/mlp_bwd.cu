@@ -27,46 +27,11 @@
 //    memory (one atomic per parameter) when the field changes.
 // kS is what shared memory holds: 64 samples at W = 64 (H <= 3), 32 at
 // W = 64 / H = 4, 128 at W = 32.
-#include "internal.cuh"
+#include "layouts.cuh"
 
 namespace roam {
 
 namespace {
-
-__host__ __device__ constexpr int round4(int x) { return (x + 3) & ~3; }
-
-// offsets of the API layout
-struct ALayout {
-    int64_t l1, hid, head, col, out, total;
-    __host__ __device__ constexpr ALayout(int W, int H)
-        : l1(0), hid((int64_t)W * kPeX + W), head(hid + (int64_t)(H - 1) * ((int64_t)W * W + W)),
-          col(head + (int64_t)(1 + W) * W + (1 + W)), out(col + (int64_t)W * (W + kPeD) + W),
-          total(out + 3 * (int64_t)W + 3)
-    {
-    }
-};
-
-// offsets of the dgrad copy: rows [out][W inputs] of the hidden layers, the
-// head's features (the density row is read from the masters) and the colour
-// layer (its F(d) inputs need no gradient)
-struct RLayout {
-    int64_t hid, head, col, total;
-    __host__ __device__ constexpr RLayout(int W, int H)
-        : hid(0), head((int64_t)(H - 1) * W * W), col(head + (int64_t)W * W), total(col + (int64_t)W * W)
-    {
-    }
-};
-
-// offsets of the transposed copy used by the forward kernel (same as mlp_simt.cu;
-// the head's row: W features, then the density logit, then zeros)
-struct TLayout {
-    int64_t l1, hid, head, col;
-    __host__ __device__ constexpr TLayout(int W, int H)
-        : l1(0), hid((int64_t)kPeX * W + W), head(hid + (int64_t)(H - 1) * ((int64_t)W * W + W)),
-          col(head + (int64_t)W * round4(1 + W) + round4(1 + W))
-    {
-    }
-};
 
 constexpr int kThreads = 256;
 constexpr int kRingRows = 16;       // weight rows per ring stage
@@ -192,7 +157,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 {
     using F = FbShape<W, H>;
     constexpr int S = F::S, XS = F::XS, KC = F::KC, NST = F::kStages;
-    constexpr ALayout A(W, H);
+    constexpr ApiLayout A(W, H);
     constexpr RLayout RL(W, H);
     constexpr TLayout TL(W, H);
     extern __shared__ float4 smem4[];
@@ -635,25 +600,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (cur != 0xffffffffu) flush(cur);
 }
 
-// API layout -> the dgrad copy (matrices only)
-__global__ void k_pack_rows(const float *__restrict__ w32, int n_fields, int W, int H, int64_t P,
-                            float *__restrict__ wr, int64_t Pr)
-{
-    const ALayout A(W, H);
-    const RLayout RL(W, H);
-    const int f = blockIdx.y;
-    const float *wf = w32 + (int64_t)f * P;
-    float *df = wr + (int64_t)f * Pr;
-    for (int q = (int)(blockIdx.x * blockDim.x + threadIdx.x); q < (int)Pr; q += (int)(gridDim.x * blockDim.x)) {
-        const int m = q / (W * W), r = q - m * W * W;
-        int64_t s;
-        if (m < H - 1) s = A.hid + (int64_t)m * (W * W + W) + r;
-        else if (m == H - 1) s = A.head + W + r;                                  // past the density row
-        else s = A.col + (int64_t)(r / W) * (W + kPeD) + r % W;
-        df[q] = wf[s];
-    }
-}
-
 __global__ void k_adam(float *__restrict__ w, float *__restrict__ m, float *__restrict__ v,
                        const float *__restrict__ g, int64_t n, float lr, float b1, float b2, float eps, float bc1,
                        float bc2)
@@ -713,8 +659,6 @@ void launch_bwd_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b
 
 bool mlp_bwd_supported(int W, int H) { return (W == 32 || W == 64) && H >= 1 && H <= 4; }
 
-int64_t rows_padded_size(int W, int H) { return RLayout(W, H).total; }
-
 int mlp_bwd_simt_tile(int W, int H)
 {
 #define ROAM_CASE(WW, HH) \
@@ -722,11 +666,6 @@ int mlp_bwd_simt_tile(int W, int H)
     ROAM_FB_CASES
 #undef ROAM_CASE
     return 128;
-}
-
-void launch_pack_rows(const float *w32, int n_fields, int W, int H, int64_t P, float *wr, int64_t Pr, cudaStream_t s)
-{
-    k_pack_rows<<<dim3((unsigned)((Pr + 1023) / 1024), (unsigned)n_fields), 256, 0, s>>>(w32, n_fields, W, H, P, wr, Pr);
 }
 
 void launch_mlp_bwd_simt(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr,

@@ -11,13 +11,11 @@
 // the head layer's loop; the 3-output colour layer is formed from the colour
 // features still in registers, the output groups' shares summed through
 // shared memory.
-#include "internal.cuh"
+#include "layouts.cuh"
 
 namespace roam {
 
 namespace {
-
-__host__ __device__ constexpr int round4(int x) { return (x + 3) & ~3; }
 
 // Thread layout of one tile: OG warps, one per output group, each over the
 // tile's 32 sample groups of 4 samples; lane l of warp og owns samples
@@ -35,23 +33,6 @@ struct SimtShape {
     static constexpr size_t kSmem = (size_t)kRows * 128 * sizeof(float) + 128 * sizeof(uint32_t);
     static_assert(TN % 4 == 0, "whole float4 runs per thread");
     static_assert(3 * OG + 1 <= kRows, "the colour sums fit in the activation buffer");
-};
-
-// Parameter offsets of the transposed copy: per layer WT[in][n_pad] then
-// bias[n_pad]; the head's row holds the W features, then the density logit
-// (column W), then zeros.
-struct TLayout {
-    int64_t l1, hid, head, col, out, total;
-    __host__ __device__ TLayout(int W, int H)
-    {
-        int64_t o = 0;
-        l1 = o;   o += (int64_t)kPeX * W + W;
-        hid = o;  o += (int64_t)(H - 1) * ((int64_t)W * W + W);
-        head = o; o += (int64_t)W * round4(1 + W) + round4(1 + W);
-        col = o;  o += (int64_t)(W + kPeD) * W + W;
-        out = o;  o += (int64_t)W * 4 + 4;
-        total = o;
-    }
 };
 
 // Weight loads: from the block's shared copy, or through the read-only path.
@@ -429,52 +410,7 @@ __global__ void __launch_bounds__(SimtSharedShape<W>::kGroups * SimtShape<W>::kT
     }
 }
 
-// API layout -> transposed copy: one thread per source parameter.
-__global__ void k_pack_simt(const float *__restrict__ w32, int n_fields, int W, int H, int64_t P,
-                            float *__restrict__ wt, int64_t Pt)
-{
-    const TLayout L(W, H);
-    const int64_t n = (int64_t)n_fields * P;
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t f = g / P;
-        int64_t q = g % P;
-        // walk the layers of the API layout: (n_out, n_in, dst offset, padded n_out)
-        int64_t dst = -1;
-        const int nl = H + 3;
-        for (int l = 0; l < nl && dst < 0; ++l) {
-            int n_out, n_in, n_pad;
-            int64_t base;
-            if (l == 0) { n_out = W; n_in = kPeX; base = L.l1; n_pad = W; }
-            else if (l < H) { n_out = W; n_in = W; base = L.hid + (int64_t)(l - 1) * (W * W + W); n_pad = W; }
-            else if (l == H) { n_out = 1 + W; n_in = W; base = L.head; n_pad = round4(1 + W); }
-            else if (l == H + 1) { n_out = W; n_in = W + kPeD; base = L.col; n_pad = W; }
-            else { n_out = 3; n_in = W; base = L.out; n_pad = 4; }
-            const int64_t nw = (int64_t)n_out * n_in;
-            // the head's output 0 (density) goes to column W, its features to 0 .. W-1
-            auto column = [&](int64_t o) { return l == H ? (o == 0 ? (int64_t)W : o - 1) : o; };
-            if (q < nw) {
-                const int64_t o = q / n_in, i = q % n_in;
-                dst = base + i * n_pad + column(o);
-            } else if (q < nw + n_out) {
-                dst = base + (int64_t)n_in * n_pad + column(q - nw);
-            } else {
-                q -= nw + n_out;
-            }
-        }
-        if (dst >= 0) wt[f * Pt + dst] = w32[g];
-    }
-}
-
 }  // namespace
-
-int64_t simt_transposed_size(int W, int H) { return TLayout(W, H).total; }
-
-void launch_pack_simt(const float *w32, int n_fields, int W, int H, int64_t P, float *wt, int64_t Pt,
-                      cudaStream_t s)
-{
-    cudaMemsetAsync(wt, 0, (size_t)n_fields * Pt * sizeof(float), s);
-    k_pack_simt<<<1024, 256, 0, s>>>(w32, n_fields, W, H, P, wt, Pt);
-}
 
 template <int W, int H>
 static void launch_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out,

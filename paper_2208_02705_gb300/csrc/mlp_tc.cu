@@ -30,6 +30,7 @@
 // s = max_k |W[n][k]| / 448, B[k][n] = e4m3(W[n][k] / s), and the epilogue
 // forms y = s * D + b.  Activations are rounded to E4M3 unscaled (the
 // ReLU/PE values of these networks sit well inside the format's range).
+#include "layouts.cuh"
 #include "tc_common.cuh"
 
 namespace roam {
@@ -414,144 +415,6 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * TcShape<W, H, F8>:
     }
 }
 
-// ---- packing: API layout -> tensor-core image ----
-
-// offsets of one field's layers in the API layout (row-major [out][in], then bias[out])
-struct ApiLayout {
-    int64_t l1, hid, head, col, out;
-    __host__ __device__ ApiLayout(int W, int H)
-    {
-        l1 = 0;
-        hid = (int64_t)W * kPeX + W;
-        head = hid + (int64_t)(H - 1) * (W * W + W);
-        col = head + (int64_t)(1 + W) * W + (1 + W);
-        out = col + (int64_t)W * (W + kPeD) + W;
-    }
-};
-
-// Weight at (n, k) of the B operand of layer l, as the MMA sees it (folded
-// bias entries included where the layout folds them).
-template <int W, int H, bool F8>
-__device__ float operand_value(const float *wf, const ApiLayout &o, int l, int n, int k)
-{
-    using S = TcShape<W, H, F8>;
-    if (k >= S::K(l)) return 0.f;
-    if (l == 0) {
-        if (n >= W) return 0.f;
-        if (k < kPeX) return wf[o.l1 + (int64_t)n * kPeX + k];
-        return (k == kPeX && !F8) ? wf[o.l1 + (int64_t)W * kPeX + n] : 0.f;
-    }
-    if (l < H) {
-        const int64_t ob = o.hid + (int64_t)(l - 1) * (W * W + W);
-        if (k < W) return wf[ob + (int64_t)n * W + k];
-        return (k == W && S::kFold) ? wf[ob + (int64_t)W * W + n] : 0.f;
-    }
-    if (l == H) {
-        // rows: W features (API rows 1..W), then the density logit (API row 0)
-        const int ar = n < W ? 1 + n : (n == W ? 0 : -1);
-        if (ar < 0) return 0.f;
-        if (k < W) return wf[o.head + (int64_t)ar * W + k];
-        return (k == W && S::kFold) ? wf[o.head + (int64_t)(1 + W) * W + ar] : 0.f;
-    }
-    const int kc = W + kPeD;
-    if (k < W) return wf[o.col + (int64_t)n * kc + k];
-    if (k == W) return F8 ? 0.f : wf[o.col + (int64_t)W * kc + n];
-    if (k <= W + kPeD) return wf[o.col + (int64_t)n * kc + (k - 1)];
-    return 0.f;
-}
-
-// bias of output n of layer l (the head's n = W is the density logit)
-template <int W, int H>
-__device__ float layer_bias(const float *wf, const ApiLayout &o, int l, int n)
-{
-    if (l == 0) return n < W ? wf[o.l1 + (int64_t)W * kPeX + n] : 0.f;
-    if (l < H) return n < W ? wf[o.hid + (int64_t)(l - 1) * (W * W + W) + (int64_t)W * W + n] : 0.f;
-    if (l == H)
-        return n < W ? wf[o.head + (int64_t)(1 + W) * W + 1 + n] : (n == W ? wf[o.head + (int64_t)(1 + W) * W] : 0.f);
-    return n < W ? wf[o.col + (int64_t)W * (W + kPeD) + n] : 0.f;
-}
-
-// per-layer FP32 table: E4M3 channel scales (max |row| / 448, 1 for an
-// all-zero row; 1 for BF16) and the biases
-template <int W, int H, bool F8>
-__global__ void k_pack_tab(const float *__restrict__ w32, int n_fields, int64_t P, uint8_t *__restrict__ img,
-                           int64_t img_bytes)
-{
-    using S = TcShape<W, H, F8>;
-    const ApiLayout o(W, H);
-    const int64_t per = (int64_t)S::kLayers * S::kTabStride;
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < (int64_t)n_fields * per;
-         g += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t f = g / per;
-        const int l = (int)((g % per) / S::kTabStride), n = (int)(g % S::kTabStride);
-        const float *wf = w32 + f * P;
-        float s = 1.f;
-        if (F8 && n < S::N(l)) {
-            float amax = 0.f;
-            for (int k = 0; k < S::K(l); ++k) amax = fmaxf(amax, fabsf(operand_value<W, H, F8>(wf, o, l, n, k)));
-            if (amax > 0.f) s = amax / 448.0f;
-        }
-        float *t = reinterpret_cast<float *>(img + f * img_bytes + S::kMatBytes + S::kOutBytes) + l * 2 * S::kTabStride;
-        t[n] = s;
-        t[S::kTabStride + n] = layer_bias<W, H>(wf, o, l, n);
-    }
-}
-
-template <int W, int H, bool F8>
-__global__ void k_pack_tc(const float *__restrict__ w32, int n_fields, int64_t P, uint8_t *__restrict__ img,
-                          int64_t img_bytes)
-{
-    using S = TcShape<W, H, F8>;
-    const ApiLayout o(W, H);
-    const int64_t per = S::kMatBytes / S::kEB;        // operand elements per field
-    const int64_t n = (int64_t)n_fields * per;
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t f = g / per;
-        const int byte = (int)((g % per) * S::kEB);
-        // find the layer and (n, k) of this element
-        int l = 0;
-        while (l + 1 < S::kLayers && byte >= S::offset(l + 1)) ++l;
-        const int lb = byte - S::offset(l);
-        const int N = S::N(l);
-        const int chunk = lb / (N * 128);
-        const int in_chunk = lb % (N * 128);
-        const int nrow = (in_chunk / 1024) * 8 + (in_chunk % 1024) / 128;
-        const int sw16 = (in_chunk % 128) / 16;
-        const int u = (sw16 ^ (nrow & 7)) & 7;               // 16-byte unit before the swizzle
-        const int k = chunk * S::kCE + u * (16 / S::kEB) + (in_chunk % 16) / S::kEB;
-        const float *wf = w32 + f * P;
-        const float v = operand_value<W, H, F8>(wf, o, l, nrow, k);
-        uint8_t *dst = img + f * img_bytes;
-        if constexpr (F8) {
-            const float s =
-                reinterpret_cast<const float *>(dst + S::kMatBytes + S::kOutBytes)[l * 2 * S::kTabStride + nrow];
-            uint16_t q;
-            asm("cvt.rn.satfinite.e4m3x2.f32 %0, %2, %1;" : "=h"(q) : "f"(v / s), "f"(0.f));
-            dst[g % per] = (uint8_t)(q & 0xffu);
-        } else {
-            const uint32_t bits = __float_as_uint(v);
-            const uint32_t r = bits + 0x7fffu + ((bits >> 16) & 1u);     // round to nearest even
-            reinterpret_cast<uint16_t *>(dst)[g % per] = (uint16_t)(r >> 16);
-        }
-    }
-    // FP32 output layer after the operands: [4][W] (weights of the 3 colours over k, a zero row), then bias[4]
-    const int nout = 4 * W + 4;
-    for (int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gi < (int64_t)n_fields * nout;
-         gi += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t f = gi / nout;
-        const int q = (int)(gi % nout);
-        const float *wf = w32 + f * P;
-        float v = 0.f;
-        if (q < 4 * W) {
-            const int c = q / W, k = q % W;
-            if (c < 3) v = wf[o.out + (int64_t)c * W + k];
-        } else if (q - 4 * W < 3) {
-            v = wf[o.out + 3 * W + (q - 4 * W)];
-        }
-        reinterpret_cast<float *>(img + f * img_bytes + S::kMatBytes)[q] = v;
-    }
-}
-
 // Where parameter q of a field (API layout) sits in its BF16 image: the byte
 // offset of its element, or -1 - r for entry r of the FP32 3-output table.
 template <int W, int H>
@@ -699,25 +562,6 @@ int tc_tile_group(int W, bool f8)
     if (W <= 32) return f8 ? TcShape<32, 1, true>::kSlots : TcShape<32, 1, false>::kSlots;
     if (W <= 64) return f8 ? TcShape<64, 1, true>::kSlots : TcShape<64, 1, false>::kSlots;
     return f8 ? TcShape<128, 1, true>::kSlots : TcShape<128, 1, false>::kSlots;
-}
-
-void launch_pack_tc(const float *w32, int n_fields, int W, int H, int64_t P, void *wimg, int64_t img_bytes, bool f8,
-                    cudaStream_t s)
-{
-#define ROAM_CASE(WW, HH)                                                                                      \
-    if (W == WW && H == HH) {                                                                                  \
-        if (f8) {                                                                                              \
-            k_pack_tab<WW, HH, true><<<1024, 256, 0, s>>>(w32, n_fields, P, (uint8_t *)wimg, img_bytes);      \
-            k_pack_tc<WW, HH, true><<<2048, 256, 0, s>>>(w32, n_fields, P, (uint8_t *)wimg, img_bytes);       \
-        } else {                                                                                               \
-            if (TcShape<WW, HH, false>::kTab)                                                                  \
-                k_pack_tab<WW, HH, false><<<1024, 256, 0, s>>>(w32, n_fields, P, (uint8_t *)wimg, img_bytes); \
-            k_pack_tc<WW, HH, false><<<2048, 256, 0, s>>>(w32, n_fields, P, (uint8_t *)wimg, img_bytes);      \
-        }                                                                                                      \
-        return;                                                                                                \
-    }
-    ROAM_TC_CASES
-#undef ROAM_CASE
 }
 
 bool launch_adam_tc(float *w32, float *m, float *v, const float *g, int n_fields, int W, int H, int64_t P, void *wimg,

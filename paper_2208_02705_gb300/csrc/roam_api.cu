@@ -305,20 +305,19 @@ roam_status refresh(roam_ctx *c, int precision, bool simt_adjoint, cudaStream_t 
 {
     for (int k = 0; k < c->n_ws; ++k) {
         WSet &q = c->ws[k];
-        if (!q.stale) continue;
-        const int H = c->md.n_hidden;
-        if ((precision == ROAM_F32 || simt_adjoint) && (q.stale & kStaleWt)) {
-            launch_pack_simt(q.w32.p, q.n, q.W, H, q.P, q.wt.p, q.Pt, s);
-            q.stale &= ~kStaleWt;
-        }
-        if (simt_adjoint && (q.stale & kStaleWr)) {
-            launch_pack_rows(q.w32.p, q.n, q.W, H, q.P, q.wr.p, q.Pr, s);
-            q.stale &= ~kStaleWr;
-        }
-        if (precision == ROAM_FP8 && (q.stale & kStaleImg8)) {
-            launch_pack_tc(q.w32.p, q.n, q.W, H, q.P, q.wimg8.p, q.img8_bytes, true, s);
-            q.stale &= ~kStaleImg8;
-        }
+        uint32_t want = 0;
+        if (precision == ROAM_F32 || simt_adjoint) want |= kStaleWt;
+        if (simt_adjoint) want |= kStaleWr;
+        if (precision == ROAM_FP8) want |= kStaleImg8;
+        want &= q.stale;
+        if (!want) continue;
+        PackDst d{};
+        if (want & kStaleWt) d.wt = q.wt.p;
+        if (want & kStaleWr) d.wr = q.wr.p;
+        if (want & kStaleImg8) d.img8 = q.wimg8.p;
+        d.img8_bytes = q.img8_bytes;
+        launch_pack(q.w32.p, q.n, q.W, c->md.n_hidden, q.P, d, s);
+        q.stale &= ~want;
         ROAM_TRY(launched("weight refresh"));
     }
     return ROAM_OK;
@@ -485,6 +484,12 @@ BucketBufs bucket_of(roam_ctx *c)
     b.sorted = c->sorted.p;
     b.tile_off = c->tile_off.p;
     return b;
+}
+
+// the training adjoint of a forward in this precision: tensor cores or SIMT
+bool adjoint_on_tc(const roam_ctx *c, int precision)
+{
+    return precision == ROAM_BF16 && mlp_bwd_tc_supported(c->md.width, c->md.n_hidden) && c->ws[0].tc_ok;
 }
 
 int tile_of(int precision) { return precision != ROAM_F32 ? tc_tile_samples() : 128; }
@@ -714,42 +719,40 @@ roam_status load_set(roam_ctx *c, int k, int W, int H, int first, int n, const f
     WSet &q = c->ws[k];
     const int64_t P = param_count(W, H);
     const int64_t total = P * n;
-    ROAM_TRY(ensure(q.w32, (size_t)total));
-    ROAM_CUDA(cudaMemcpy(q.w32.p, weights, total * sizeof(float),
-                         on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice));
-    ROAM_CUDA(cudaMemset(c->d_flag, 0, 4));
-    k_check_finite<<<1024, 256>>>(q.w32.p, total, c->d_flag);
-    ROAM_TRY(launched("weight check"));
-    uint32_t bad = 0;
-    ROAM_CUDA(cudaMemcpy(&bad, c->d_flag, 4, cudaMemcpyDeviceToHost));
-    if (bad) return fail(ROAM_ERR_ARG, "weights contain NaN or Inf");
     q.W = W;
     q.first = first;
     q.n = n;
     q.P = P;
     q.stale = 0;
     q.Pt = simt_transposed_size(W, H);
-    ROAM_TRY(ensure(q.wt, (size_t)(q.Pt * n)));
-    launch_pack_simt(q.w32.p, n, W, H, P, q.wt.p, q.Pt, 0);
-    ROAM_TRY(launched("pack simt"));
     q.Pr = rows_padded_size(W, H);
-    ROAM_TRY(ensure(q.wr, (size_t)(q.Pr * n)));
-    launch_pack_rows(q.w32.p, n, W, H, P, q.wr.p, q.Pr, 0);
-    ROAM_TRY(launched("pack rows"));
     q.tc_ok = tc_supported(W, H, false);
-    if (q.tc_ok) {
-        q.img_bytes = tc_image_bytes(W, H, false);
-        ROAM_TRY(ensure(q.wimg, (size_t)(q.img_bytes * n)));
-        launch_pack_tc(q.w32.p, n, W, H, P, q.wimg.p, q.img_bytes, false, 0);
-        ROAM_TRY(launched("pack tc"));
-    }
     q.tc8_ok = tc_supported(W, H, true);
-    if (q.tc8_ok) {
-        q.img8_bytes = tc_image_bytes(W, H, true);
-        ROAM_TRY(ensure(q.wimg8, (size_t)(q.img8_bytes * n)));
-        launch_pack_tc(q.w32.p, n, W, H, P, q.wimg8.p, q.img8_bytes, true, 0);
-        ROAM_TRY(launched("pack tc fp8"));
-    }
+    q.img_bytes = q.tc_ok ? tc_image_bytes(W, H, false) : 0;
+    q.img8_bytes = q.tc8_ok ? tc_image_bytes(W, H, true) : 0;
+    ROAM_TRY(ensure(q.w32, (size_t)total));
+    ROAM_TRY(ensure(q.wt, (size_t)(q.Pt * n)));
+    ROAM_TRY(ensure(q.wr, (size_t)(q.Pr * n)));
+    if (q.tc_ok) ROAM_TRY(ensure(q.wimg, (size_t)(q.img_bytes * n)));
+    if (q.tc8_ok) ROAM_TRY(ensure(q.wimg8, (size_t)(q.img8_bytes * n)));
+    // device weights are read once, by the pass that writes the masters and
+    // every copy of them
+    if (!on_device) ROAM_CUDA(cudaMemcpy(q.w32.p, weights, total * sizeof(float), cudaMemcpyHostToDevice));
+    PackDst d{};
+    d.w32 = on_device ? q.w32.p : nullptr;
+    d.wt = q.wt.p;
+    d.wr = q.wr.p;
+    d.img = q.tc_ok ? q.wimg.p : nullptr;
+    d.img8 = q.tc8_ok ? q.wimg8.p : nullptr;
+    d.img_bytes = q.img_bytes;
+    d.img8_bytes = q.img8_bytes;
+    d.bad = c->d_flag;
+    ROAM_CUDA(cudaMemset(c->d_flag, 0, 4));
+    launch_pack(on_device ? weights : q.w32.p, n, W, H, P, d, 0);
+    ROAM_TRY(launched("weight pack"));
+    uint32_t bad = 0;
+    ROAM_CUDA(cudaMemcpy(&bad, c->d_flag, 4, cudaMemcpyDeviceToHost));
+    if (bad) return fail(ROAM_ERR_ARG, "weights contain NaN or Inf");
     return ROAM_OK;
 }
 
@@ -1605,10 +1608,11 @@ roam_status roam_train_forward(roam_ctx *c, const roam_camera *cams, int n_views
     // finds each ray's samples in one place
     const int R = opts->n_max;
     if ((double)((n_rays + 31) & ~31LL) * R >= 4294967295.0) return fail(ROAM_ERR_ARG, "too many rays x samples");
-    ROAM_TRY(ensure_rays(c, n_rays, R));
     // (the SIMT adjoint's tiles may be smaller than the forward's)
-    ROAM_TRY(ensure(c->tiles, tile_capacity(c, (size_t)((n_rays + 31) & ~31LL) * (size_t)R,
-                                            mlp_bwd_simt_tile(c->md.width, c->md.n_hidden))));
+    if (!adjoint_on_tc(c, opts->precision))
+        ROAM_TRY(ensure(c->tiles, tile_capacity(c, (size_t)((n_rays + 31) & ~31LL) * (size_t)R,
+                                                mlp_bwd_simt_tile(c->md.width, c->md.n_hidden))));
+    ROAM_TRY(ensure_rays(c, n_rays, R));
     ROAM_CUDA(cudaMemsetAsync(c->ctr, 0, sizeof(Counters), s));
     ROAM_CUDA(cudaMemsetAsync(c->hist.p, 0, (size_t)c->n_fields * sizeof(uint32_t), s));
     ROAM_TRY(run_rounds(c, rays, n_rays, opts, rgb, nullptr, nullptr, R, R, s));
@@ -1645,7 +1649,7 @@ roam_status roam_train_backward(roam_ctx *c, const float *dl_drgb, float *grad, 
     ROAM_TRY(launched("composite_bwd"));
     ROAM_CUDA(cudaMemsetAsync(c->aux, 0, sizeof(Counters), s));
     const BucketBufs b = bucket_of(c);
-    const bool tc = o.precision == ROAM_BF16 && mlp_bwd_tc_supported(c->md.width, c->md.n_hidden) && c->ws[0].tc_ok;
+    const bool tc = adjoint_on_tc(c, o.precision);
     const int tile = tc ? 128 : mlp_bwd_simt_tile(c->md.width, c->md.n_hidden);
     {
         ProfScope ps(c, P_BUCKET, s);
@@ -1725,7 +1729,12 @@ roam_status roam_adam_step(roam_ctx *c, const float *grad, const roam_adam_cfg *
         if (!fused) {
             launch_adam(q.w32.p, c->adam_m.p, c->adam_v.p, grad, n, cfg->lr, cfg->beta1, cfg->beta2, cfg->eps, bc1,
                         bc2, s);
-            if (q.tc_ok) launch_pack_tc(q.w32.p, c->n_fields, W, H, q.P, q.wimg.p, q.img_bytes, false, s);
+            if (q.tc_ok) {
+                PackDst d{};
+                d.img = q.wimg.p;
+                d.img_bytes = q.img_bytes;
+                launch_pack(q.w32.p, c->n_fields, W, H, q.P, d, s);
+            }
         }
         q.stale |= kStaleWt | kStaleWr | (q.tc8_ok ? kStaleImg8 : 0u);
         if (!q.tc_ok) ROAM_TRY(refresh(c, ROAM_F32, true, s));
