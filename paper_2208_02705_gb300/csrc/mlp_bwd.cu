@@ -27,7 +27,11 @@
 //    memory (one atomic per parameter) when the field changes.
 // kS is what shared memory holds: 64 samples at W = 64 (H <= 3), 32 at
 // W = 64 / H = 4, 128 at W = 32.
+#include <cooperative_groups.h>
+
 #include "layouts.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace roam {
 
@@ -615,31 +619,66 @@ __global__ void k_adam(float *__restrict__ w, float *__restrict__ m, float *__re
     }
 }
 
-// L2 photometric loss of the fine-tuning stage: loss += sum (rgb - target)^2
-// / norm over the rays, and dl/drgb = 2 (rgb - target) / norm.
-// One block: the loss is summed in a fixed order (per-thread strided sums,
-// then a fixed tree), so the same inputs give the same bits on every run.
-__global__ void __launch_bounds__(1024) k_l2_loss(int64_t n3, const float *__restrict__ rgb,
-                                                  const float *__restrict__ target, float inv_norm,
-                                                  float *__restrict__ dl, float *__restrict__ loss)
+// The losses: one cluster of 8 blocks, the sum in a fixed order (per-thread
+// strided sums, a fixed tree over the warp, the block and then the cluster,
+// through distributed shared memory), so the same inputs give the same bits on
+// every run, without scratch memory or a second launch.  One block alone took
+// 34 us for 65,536 rays: its 32 warps cannot keep enough loads in flight.
+constexpr int kLossBlocks = 8;
+
+// every thread's sum over the cluster, in block 0's thread 0
+__device__ __forceinline__ float cluster_sum(float acc)
 {
     __shared__ float part[32];
-    float acc = 0.f;
-    for (int64_t i = threadIdx.x; i < n3; i += blockDim.x) {
-        const float e = rgb[i] - target[i];
-        dl[i] = 2.f * e * inv_norm;
-        acc = fmaf(e * inv_norm, e, acc);
-    }
+    cg::cluster_group cluster = cg::this_cluster();
+    const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+    if (lane == 0) part[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x < 32) {
-        float v = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.f;
+        acc = part[lane];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0 && loss) *loss = v;
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        if (lane == 0) part[0] = acc;
     }
+    cluster.sync();
+    float v = 0.f;
+    if (cluster.block_rank() == 0 && threadIdx.x == 0)
+        for (int q = 0; q < kLossBlocks; ++q) v += cluster.map_shared_rank(part, q)[0];
+    cluster.sync();                                   // no block leaves while its sum is read
+    return v;
+}
+
+// L2 photometric loss of the fine-tuning stage: loss = sum (rgb - target)^2
+// / norm over the rays, and dl/drgb = 2 (rgb - target) / norm (kVec: the three
+// arrays are 16-byte aligned).
+template <bool kVec>
+__global__ void __cluster_dims__(kLossBlocks, 1, 1) __launch_bounds__(1024)
+    k_l2_loss(int64_t n3, const float *__restrict__ rgb, const float *__restrict__ target, float inv_norm,
+              float *__restrict__ dl, float *__restrict__ loss)
+{
+    float acc = 0.f;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    auto one = [&](float a, float b) {
+        const float e = a - b;
+        acc = fmaf(e * inv_norm, e, acc);
+        return 2.f * e * inv_norm;
+    };
+    const int64_t n4 = kVec ? n3 / 4 : 0;
+#pragma unroll 4
+    for (int64_t i = t; i < n4; i += stride) {
+        const float4 a = reinterpret_cast<const float4 *>(rgb)[i], b = reinterpret_cast<const float4 *>(target)[i];
+        float4 d;
+        d.x = one(a.x, b.x);
+        d.y = one(a.y, b.y);
+        d.z = one(a.z, b.z);
+        d.w = one(a.w, b.w);
+        reinterpret_cast<float4 *>(dl)[i] = d;
+    }
+    for (int64_t i = 4 * n4 + t; i < n3; i += stride) dl[i] = one(rgb[i], target[i]);
+    acc = cluster_sum(acc);
+    if (t == 0 && loss) *loss = acc;
 }
 
 template <int W, int H>
@@ -678,14 +717,15 @@ void launch_mlp_bwd_simt(const MlpWeights &w, const SampleSrc &src, const Bucket
 }
 
 // Eq. 7 over samples: sum [(sigma_s - sigma_t)^2 + |c_s - c_t|^2] / I, its
-// gradient 2 (student - teacher) / I per component; one block, fixed order.
-__global__ void __launch_bounds__(1024) k_distill_loss(int64_t n, const float4 *__restrict__ st,
-                                                       const float4 *__restrict__ te, float inv_I,
-                                                       float4 *__restrict__ dl, float *__restrict__ loss)
+// gradient 2 (student - teacher) / I per component.
+__global__ void __cluster_dims__(kLossBlocks, 1, 1) __launch_bounds__(1024)
+    k_distill_loss(int64_t n, const float4 *__restrict__ st, const float4 *__restrict__ te, float inv_I,
+                   float4 *__restrict__ dl, float *__restrict__ loss)
 {
-    __shared__ float part[32];
     float acc = 0.f;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll 4
+    for (int64_t i = t; i < n; i += stride) {
         const float4 a = st[i], b = te[i];
         const float e0 = a.x - b.x, e1 = a.y - b.y, e2 = a.z - b.z, e3 = a.w - b.w;
         dl[i] = make_float4(2.f * e0 * inv_I, 2.f * e1 * inv_I, 2.f * e2 * inv_I, 2.f * e3 * inv_I);
@@ -694,28 +734,21 @@ __global__ void __launch_bounds__(1024) k_distill_loss(int64_t n, const float4 *
         acc = fmaf(e2 * inv_I, e2, acc);
         acc = fmaf(e3 * inv_I, e3, acc);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0 && loss) *loss = v;
-    }
+    acc = cluster_sum(acc);
+    if (t == 0 && loss) *loss = acc;
 }
 
 void launch_distill_loss(int64_t n, const float4 *student, const float4 *teacher, float I, float4 *dl, float *loss,
                          cudaStream_t s)
 {
-    k_distill_loss<<<1, 1024, 0, s>>>(n, student, teacher, 1.0f / I, dl, loss);
+    k_distill_loss<<<kLossBlocks, 1024, 0, s>>>(n, student, teacher, 1.0f / I, dl, loss);
 }
 
 void launch_l2_loss(int64_t n_rays, const float *rgb, const float *target, float norm, float *dl, float *loss,
                     cudaStream_t s)
 {
-    k_l2_loss<<<1, 1024, 0, s>>>(3 * n_rays, rgb, target, 1.0f / norm, dl, loss);
+    const bool vec = (((uintptr_t)rgb | (uintptr_t)target | (uintptr_t)dl) & 15) == 0;
+    (vec ? k_l2_loss<true> : k_l2_loss<false>)<<<kLossBlocks, 1024, 0, s>>>(3 * n_rays, rgb, target, 1.0f / norm, dl, loss);
 }
 
 void launch_adam(float *w32, float *m, float *v, const float *g, int64_t n, float lr, float b1, float b2, float eps,
