@@ -50,6 +50,7 @@ struct GridDev {
     float vox, inv_vox;
     const uint32_t *bits;         // [gz][gy][wpr]
     const uint32_t *prefix;       // exclusive popcount before each word
+    const uint2 *cells;           // the two side by side: (word, prefix)
     const uint8_t *brick_dist;    // [bz][by][bx] Chebyshev distance (bricks) to an occupied brick, 0 = occupied
     const uint16_t *labels;       // field of each occupied voxel, rank order
     int n_fields;
@@ -224,7 +225,7 @@ struct MlpWeights {
 
 // ---- kernels launched from the API layer -------------------------------
 
-void launch_grid_prefix(const uint32_t *bits, uint32_t *prefix, uint32_t *block_sums,
+void launch_grid_prefix(const uint32_t *bits, uint32_t *prefix, uint32_t *block_sums, uint2 *cells,
                         int64_t n_words, cudaStream_t s);
 void launch_brick_dist(GridDev g, uint8_t *occ, uint16_t *t0, uint16_t *t1, uint8_t *dist, cudaStream_t s);
 void launch_march(const GridDev &g, const MarchParams &p, int grid, cudaStream_t s);

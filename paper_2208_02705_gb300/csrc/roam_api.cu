@@ -114,6 +114,7 @@ struct roam_ctx {
     GridDev g{};
     int64_t n_words = 0, n_occ = 0;
     DBuf<uint32_t> bits, prefix, block_sums;
+    DBuf<uint2> cells;
     DBuf<uint8_t> brick_occ, brick_dist;
     DBuf<uint16_t> brick_t0, brick_t1;
     // fields
@@ -820,7 +821,7 @@ roam_status roam_destroy(roam_ctx *c)
     if (!c) return ROAM_OK;
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
-    release(c->bits); release(c->prefix); release(c->block_sums);
+    release(c->bits); release(c->prefix); release(c->cells); release(c->block_sums);
     release(c->brick_occ); release(c->brick_dist); release(c->brick_t0); release(c->brick_t1);
     release(c->labels); release(c->affine);
     for (WSet &q : c->ws) {
@@ -878,6 +879,7 @@ roam_status roam_load_grid(roam_ctx *c, const roam_grid_desc *desc, const uint32
     const int64_t n_words = (int64_t)desc->dims[0] / 32 * desc->dims[1] * desc->dims[2];
     ROAM_TRY(ensure(c->bits, (size_t)n_words));
     ROAM_TRY(ensure(c->prefix, (size_t)n_words));
+    ROAM_TRY(ensure(c->cells, (size_t)n_words));
     ROAM_TRY(ensure(c->block_sums, (size_t)((n_words + 4095) / 4096)));
     ROAM_CUDA(cudaMemcpy(c->bits.p, bits, n_words * sizeof(uint32_t),
                          on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice));
@@ -895,10 +897,11 @@ roam_status roam_load_grid(roam_ctx *c, const roam_grid_desc *desc, const uint32
     ROAM_TRY(ensure(c->brick_t1, n_bricks));
     g.bits = c->bits.p;
     g.prefix = c->prefix.p;
+    g.cells = c->cells.p;
     g.brick_dist = c->brick_dist.p;
     g.labels = nullptr;
     g.n_fields = 0;
-    launch_grid_prefix(c->bits.p, c->prefix.p, c->block_sums.p, n_words, 0);
+    launch_grid_prefix(c->bits.p, c->prefix.p, c->block_sums.p, c->cells.p, n_words, 0);
     ROAM_TRY(launched("grid prefix"));
     launch_brick_dist(g, c->brick_occ.p, c->brick_t0.p, c->brick_t1.p, c->brick_dist.p, 0);
     ROAM_TRY(launched("brick distance map"));
