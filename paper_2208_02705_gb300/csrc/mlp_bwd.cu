@@ -29,7 +29,7 @@
 // W = 64 / H = 4, 128 at W = 32.
 #include <cooperative_groups.h>
 
-#include "layouts.cuh"
+#include "simt_common.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -83,77 +83,6 @@ struct FbShape {
     static_assert(kStages >= 4, "the weight ring keeps a few stages in flight");
     static_assert(TN == 2 || TN == 4, "forward tiles of 2 or 4 outputs");
 };
-
-__device__ __forceinline__ float local_coord(float th0, float delta, float o, float dh, float dl, float scale,
-                                             float offset)
-{
-    const float t_hi = __fmul_rn(th0, delta);
-    const float t_lo = __fmaf_rn(th0, delta, -t_hi);
-    const float ph = __fmul_rn(t_hi, dh);
-    const float pl = __fadd_rn(__fmaf_rn(t_hi, dh, -ph), __fadd_rn(__fmul_rn(t_hi, dl), __fmul_rn(t_lo, dh)));
-    const float sh = __fadd_rn(o, ph);
-    const float bv = __fsub_rn(sh, o);
-    const float se = __fadd_rn(__fsub_rn(o, __fsub_rn(sh, bv)), __fsub_rn(ph, bv));
-    const float sl = __fadd_rn(se, pl);
-    const float qh = __fmul_rn(scale, sh);
-    const float ql = __fadd_rn(__fmaf_rn(scale, sh, -qh), __fmul_rn(scale, sl));
-    return __fadd_rn(__fadd_rn(qh, offset), ql);
-}
-
-__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-
-// TN consecutive floats from shared memory
-template <int TN>
-__device__ __forceinline__ void ld_row(const float *p, float2 (&w)[TN / 2])
-{
-    if constexpr (TN >= 4) {
-#pragma unroll
-        for (int q = 0; q < TN / 4; ++q) {
-            const float4 v = *reinterpret_cast<const float4 *>(p + 4 * q);
-            w[2 * q] = make_float2(v.x, v.y);
-            w[2 * q + 1] = make_float2(v.z, v.w);
-        }
-    } else {
-        w[0] = *reinterpret_cast<const float2 *>(p);
-    }
-}
-
-// One tile's sample of this thread (thread t of a group of kS takes sample
-// t mod kS), gathered in stages a tile ahead so that no stage waits for the
-// load before it.
-struct FbPending {
-    bool on;
-    uint32_t idx, rec, ray;
-    float4 o, d, dl;
-};
-
-__device__ __forceinline__ void fb_index(FbPending &q, const BucketBufs &b, const Tile &tl, int s, bool more)
-{
-    q.on = more && (uint32_t)s < tl.count;
-    if (q.on) q.idx = b.sorted[tl.start + s];
-}
-
-__device__ __forceinline__ void fb_record(FbPending &q, const SampleSrc &src)
-{
-    if (!q.on || src.mode != 0) return;
-    const uint32_t i = group_of(q.idx >> 5, (uint32_t)src.R) * 32u + (q.idx & 31u);
-    q.rec = src.recs[q.idx];
-    q.ray = src.live ? src.live[i] : i;
-}
-
-__device__ __forceinline__ void fb_ray(FbPending &q, const SampleSrc &src)
-{
-    if (!q.on) return;
-    if (src.mode == 0) {
-        q.o = src.st.orig[q.ray];
-        q.d = src.st.dir[q.ray];
-        if (src.accurate) q.dl = src.st.dir_lo[q.ray];
-    } else {
-        const int64_t k = 3 * (int64_t)q.idx;
-        q.o = make_float4(src.p[k], src.p[k + 1], src.p[k + 2], 0.f);
-        q.d = make_float4(src.d[k], src.d[k + 1], src.d[k + 2], 0.f);
-    }
-}
 
 template <int W, int H>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -376,16 +305,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int smp = tid % S;                     // this thread's sample in the gather and the encoding
     constexpr int NP = kThreads / S;             // threads per sample
     const int part = tid / S;
-    FbPending pend{};
+    SimtPending pend{};
     if (t0 < t1) {
         tl = b.tiles[t0];
-        fb_index(pend, b, tl, smp, true);
-        fb_record(pend, src);
-        fb_ray(pend, src);
+        simt_index(pend, b, tl, smp, true);
+        simt_record(pend, src);
+        simt_ray(pend, src);
     }
     for (uint32_t t = t0; t < t1; ++t) {
         const Tile tc = tl;
-        const FbPending me = pend;
+        const SimtPending me = pend;
         const bool more = t + 1 < t1;
         if (more) tl = b.tiles[t + 1];
         // (every thread is past the previous tile's last reads: the barrier below)
@@ -410,42 +339,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         // ---- encode: the sample's frequencies split over its NP threads ----
         const float4 gv = me.on ? gsr[me.idx] : make_float4(0.f, 0.f, 0.f, 0.f);
-        {
-            const float *aff = w.affine + 6 * (int64_t)tc.field;
-            float xl[3] = {0.f, 0.f, 0.f}, dv[3] = {0.f, 0.f, 1.f};
-            if (me.on) {
-                const float op[3] = {me.o.x, me.o.y, me.o.z}, dp[3] = {me.d.x, me.d.y, me.d.z},
-                            lp[3] = {me.dl.x, me.dl.y, me.dl.z};
-                const float th0 = (float)(me.rec & 0xffffu) + 0.5f;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    dv[a] = dp[a];
-                    if (src.mode == 1) xl[a] = fmaf(aff[a], op[a], aff[3 + a]);
-                    else if (src.accurate) xl[a] = local_coord(th0, src.delta, op[a], dp[a], lp[a], aff[a], aff[3 + a]);
-                    else xl[a] = fmaf(aff[a], fmaf(th0 * src.delta, dp[a], op[a]), aff[3 + a]);
-                }
-            }
-            float *xp = X + F::rX * XS + smp, *dp = X + (F::rC + W) * XS + smp;
-            if (part == 0) {
-#pragma unroll
-                for (int a = 0; a < 3; ++a) xp[a * XS] = xl[a];
-            } else if (part == 1) {
-#pragma unroll
-                for (int a = 0; a < 3; ++a) dp[a * XS] = dv[a];
-            }
-            for (int k = part; k < 14; k += NP) {
-                const bool pos = k < 10;
-                const int kk = pos ? k : k - 10;
-                float *row = (pos ? xp : dp) + (3 + 6 * kk) * XS;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    float s, c;
-                    sincospif(ldexpf(pos ? xl[a] : dv[a], kk), &s, &c);
-                    row[a * XS] = s;
-                    row[(3 + a) * XS] = c;
-                }
-            }
-        }
+        simt_encode<NP, XS>(me, src, w.affine + 6 * (int64_t)tc.field, X + F::rX * XS + smp, X + (F::rC + W) * XS + smp,
+                            part);
         sync();
 
         // ---- forward recompute ----
@@ -462,14 +357,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             sync();
         };
         forward(Int<kPeX>{}, Int<W>{}, 0, X + F::rX * XS, X + F::rH(1) * XS, true);
-        fb_index(pend, b, tl, smp, more);
+        simt_index(pend, b, tl, smp, more);
 #pragma unroll 1
         for (int l = 1; l < H; ++l)
             forward(Int<W>{}, Int<W>{}, l, X + F::rH(l) * XS, X + F::rH(l + 1) * XS, true);
         forward(Int<W>{}, Int<F::NH>{}, H, X + F::rH(H) * XS, X + F::rC * XS, false);
-        fb_record(pend, src);
+        simt_record(pend, src);
         forward(Int<KC>{}, Int<W>{}, H + 1, X + F::rC * XS, X + F::rG * XS, true);
-        fb_ray(pend, src);
+        simt_ray(pend, src);
 
         // ---- outputs and the loss gradient at their logits: rgb by parts
         // 0 .. 2, the density by part 3 (a sample's parts go round its threads) ----
