@@ -61,12 +61,12 @@ struct AssignState {
     uint32_t done;               // blocks finished in the current launch (the last one does the serial part)
 };
 
-__global__ void k_occupied_list(const uint32_t *bits, const uint32_t *prefix, int64_t n_words, uint32_t *vox)
+__global__ void k_occupied_list(const uint2 *cells, int64_t n_words, uint32_t *vox)
 {
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n_words;
          w += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t word = bits[w];
-        uint32_t r = prefix[w];
+        const uint2 cell = cells[w];
+        uint32_t word = cell.x, r = cell.y;
         while (word) {
             const int b = __ffs(word) - 1;
             vox[r++] = (uint32_t)(w * 32 + b);
@@ -297,8 +297,7 @@ struct BrickLists {
 
 // one warp per brick: its occupied voxels, appended to the lists (bricks in
 // any order: the networks do not depend on it)
-__global__ void __launch_bounds__(256) k_brick_lists(const uint32_t *__restrict__ bits, const uint32_t *__restrict__ prefix,
-                                                     int gx, int gy, int gz, BrickLists L)
+__global__ void __launch_bounds__(256) k_brick_lists(const uint2 *__restrict__ cells, int gx, int gy, int gz, BrickLists L)
 {
     const int bx_n = gx >> 3, by_n = gy >> 3, bz_n = gz >> 3, wpr = gx >> 5, lane = threadIdx.x & 31;
     const uint32_t n_b = (uint32_t)bx_n * by_n * bz_n;
@@ -310,9 +309,10 @@ __global__ void __launch_bounds__(256) k_brick_lists(const uint32_t *__restrict_
         for (int h = 0; h < 2; ++h) {
             const int r = lane + 32 * h, y = by * 8 + (r & 7), z = bz * 8 + (r >> 3);     // row r of the brick
             const uint32_t w = ((uint32_t)z * gy + y) * wpr + (bx >> 2);
-            const uint32_t word = bits[w], sh = (uint32_t)(bx & 3) * 8;
-            m[h] = (word >> sh) & 0xffu;
-            base[h] = prefix[w] + (uint32_t)__popc(word & ((1u << sh) - 1u));
+            const uint2 cell = cells[w];
+            const uint32_t sh = (uint32_t)(bx & 3) * 8;
+            m[h] = (cell.x >> sh) & 0xffu;
+            base[h] = cell.y + (uint32_t)__popc(cell.x & ((1u << sh) - 1u));
             own += __popc(m[h]);
         }
         int incl = own;
@@ -616,7 +616,7 @@ size_t assign_scratch_bytes(uint32_t S, int64_t n_bricks)
     return sizeof(AssignState) + kBins * sizeof(uint32_t) + 16 + nb * 12 + (size_t)S * 6;
 }
 
-void launch_assign(const uint32_t *bits, const uint32_t *prefix, int64_t n_words, int gx, int gy, int gz, uint32_t S,
+void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, uint32_t S,
                    int n, uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm, cudaStream_t s)
 {
     AssignState *st = reinterpret_cast<AssignState *>(scratch);
@@ -624,7 +624,7 @@ void launch_assign(const uint32_t *bits, const uint32_t *prefix, int64_t n_words
     // (16 more bytes: the lists' two counters)
     cudaMemsetAsync(scratch, 0, sizeof(AssignState) + kBins * sizeof(uint32_t) + 16, s);
     cudaMemsetAsync(field, 0xff, (size_t)S * sizeof(uint16_t), s);
-    k_occupied_list<<<n_sm * 8, 256, 0, s>>>(bits, prefix, n_words, vox);
+    k_occupied_list<<<n_sm * 8, 256, 0, s>>>(cells, n_words, vox);
     const uint32_t per = S / (uint32_t)n;
     const int grid = n_sm * 4;
     if (n > 1 && per <= kBrickMaxPer) {
@@ -637,7 +637,7 @@ void launch_assign(const uint32_t *bits, const uint32_t *prefix, int64_t n_words
         L.start = L.count + nb;
         L.rank = L.start + nb;
         L.loc = reinterpret_cast<uint16_t *>(L.rank + S);
-        k_brick_lists<<<n_sm * 8, 256, 0, s>>>(bits, prefix, gx, gy, gz, L);
+        k_brick_lists<<<n_sm * 8, 256, 0, s>>>(cells, gx, gy, gz, L);
         k_assign_bricks<<<kCluster, kAT, 0, s>>>(field, S, vox, gx, gy, st, L, n, per);
     } else if (n > 1) {
         // per network: 4 digit passes (histogram, then the select in the block

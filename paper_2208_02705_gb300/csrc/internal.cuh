@@ -49,8 +49,7 @@ struct GridDev {
     float origin[3];
     float vox, inv_vox;
     const uint32_t *bits;         // [gz][gy][wpr]
-    const uint32_t *prefix;       // exclusive popcount before each word
-    const uint2 *cells;           // the two side by side: (word, prefix)
+    const uint2 *cells;           // (word, exclusive popcount before it), side by side for the march
     const uint8_t *brick_dist;    // [bz][by][bx] Chebyshev distance (bricks) to an occupied brick, 0 = occupied
     const uint16_t *labels;       // field of each occupied voxel, rank order
     int n_fields;
@@ -225,8 +224,7 @@ struct MlpWeights {
 
 // ---- kernels launched from the API layer -------------------------------
 
-void launch_grid_prefix(const uint32_t *bits, uint32_t *prefix, uint32_t *block_sums, uint2 *cells,
-                        int64_t n_words, cudaStream_t s);
+void launch_grid_cells(const uint32_t *bits, uint2 *cells, uint32_t *block_sums, int64_t n_words, cudaStream_t s);
 void launch_brick_dist(GridDev g, uint8_t *occ, uint16_t *t0, uint16_t *t1, uint8_t *dist, cudaStream_t s);
 void launch_march(const GridDev &g, const MarchParams &p, int grid, cudaStream_t s);
 struct TeacherAffine {
@@ -244,7 +242,7 @@ void launch_teacher_simt(const float *wt, TeacherAffine aff, int64_t n, const fl
 void launch_distill_loss(int64_t n, const float4 *student, const float4 *teacher, float I, float4 *dl, float *loss,
                          cudaStream_t s);
 size_t assign_scratch_bytes(uint32_t S, int64_t n_bricks);
-void launch_assign(const uint32_t *bits, const uint32_t *prefix, int64_t n_words, int gx, int gy, int gz, uint32_t S,
+void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, uint32_t S,
                    int n, uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm, cudaStream_t s);
 uint32_t assign_status(const void *scratch);
 size_t occupancy_view_bytes(int n_views);

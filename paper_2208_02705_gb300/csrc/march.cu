@@ -40,23 +40,23 @@ __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *total)
     return excl;
 }
 
-// prefix[w] = popcount of all words before w, in blocks of 4096 words
-__global__ void k_prefix_local(const uint32_t *__restrict__ bits, uint32_t *__restrict__ prefix,
+// cells[w] = (word w, popcount of all words before w), in blocks of 4096 words
+__global__ void k_prefix_local(const uint32_t *__restrict__ bits, uint2 *__restrict__ cells,
                                uint32_t *__restrict__ block_sums, int64_t n_words)
 {
     const int64_t base = (int64_t)blockIdx.x * 4096 + threadIdx.x * 4;
-    uint32_t c[4], s = 0;
+    uint32_t w[4], s = 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        c[q] = base + q < n_words ? (uint32_t)__popc(bits[base + q]) : 0u;
-        s += c[q];
+        w[q] = base + q < n_words ? bits[base + q] : 0u;
+        s += (uint32_t)__popc(w[q]);
     }
     uint32_t tot;
     uint32_t e = block_exclusive_scan(s, &tot);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        if (base + q < n_words) prefix[base + q] = e;
-        e += c[q];
+        if (base + q < n_words) cells[base + q] = make_uint2(w[q], e);
+        e += (uint32_t)__popc(w[q]);
     }
     if (threadIdx.x == 0) block_sums[blockIdx.x] = tot;
 }
@@ -74,15 +74,10 @@ __global__ void k_prefix_blocks(uint32_t *block_sums, int64_t n_blocks)
     }
 }
 
-// ... and each word beside its prefix, as the march reads them (one load)
-__global__ void k_prefix_add(const uint32_t *bits, uint32_t *prefix, const uint32_t *block_sums, uint2 *cells,
-                             int64_t n_words)
+__global__ void k_prefix_add(uint2 *cells, const uint32_t *block_sums, int64_t n_words)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_words) return;
-    const uint32_t p = prefix[i] + block_sums[i / 4096];
-    prefix[i] = p;
-    cells[i] = make_uint2(bits[i], p);
+    if (i < n_words) cells[i].y += block_sums[i / 4096];
 }
 
 // one thread per 8^3 brick: 1 if any of its 512 voxels is occupied
@@ -430,13 +425,12 @@ __global__ void __launch_bounds__(256) k_march(GridDev g, MarchParams p)
 
 }  // namespace
 
-void launch_grid_prefix(const uint32_t *bits, uint32_t *prefix, uint32_t *block_sums, uint2 *cells, int64_t n_words,
-                        cudaStream_t s)
+void launch_grid_cells(const uint32_t *bits, uint2 *cells, uint32_t *block_sums, int64_t n_words, cudaStream_t s)
 {
     const int64_t nb = (n_words + 4095) / 4096;
-    k_prefix_local<<<(unsigned)nb, 1024, 0, s>>>(bits, prefix, block_sums, n_words);
+    k_prefix_local<<<(unsigned)nb, 1024, 0, s>>>(bits, cells, block_sums, n_words);
     k_prefix_blocks<<<1, 1024, 0, s>>>(block_sums, nb);
-    k_prefix_add<<<(unsigned)((n_words + 255) / 256), 256, 0, s>>>(bits, prefix, block_sums, cells, n_words);
+    k_prefix_add<<<(unsigned)((n_words + 255) / 256), 256, 0, s>>>(cells, block_sums, n_words);
 }
 
 void launch_brick_dist(GridDev g, uint8_t *occ, uint16_t *t0, uint16_t *t1, uint8_t *dist, cudaStream_t s)

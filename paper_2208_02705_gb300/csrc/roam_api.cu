@@ -113,8 +113,8 @@ struct roam_ctx {
     roam_grid_desc gd{};
     GridDev g{};
     int64_t n_words = 0, n_occ = 0;
-    DBuf<uint32_t> bits, prefix, block_sums;
-    DBuf<uint2> cells;
+    DBuf<uint32_t> bits, block_sums;
+    DBuf<uint2> cells;                      // the bit words beside their rank prefixes
     DBuf<uint8_t> brick_occ, brick_dist;
     DBuf<uint16_t> brick_t0, brick_t1;
     // fields
@@ -821,7 +821,7 @@ roam_status roam_destroy(roam_ctx *c)
     if (!c) return ROAM_OK;
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
-    release(c->bits); release(c->prefix); release(c->cells); release(c->block_sums);
+    release(c->bits); release(c->cells); release(c->block_sums);
     release(c->brick_occ); release(c->brick_dist); release(c->brick_t0); release(c->brick_t1);
     release(c->labels); release(c->affine);
     for (WSet &q : c->ws) {
@@ -878,7 +878,6 @@ roam_status roam_load_grid(roam_ctx *c, const roam_grid_desc *desc, const uint32
     ++c->gen;
     const int64_t n_words = (int64_t)desc->dims[0] / 32 * desc->dims[1] * desc->dims[2];
     ROAM_TRY(ensure(c->bits, (size_t)n_words));
-    ROAM_TRY(ensure(c->prefix, (size_t)n_words));
     ROAM_TRY(ensure(c->cells, (size_t)n_words));
     ROAM_TRY(ensure(c->block_sums, (size_t)((n_words + 4095) / 4096)));
     ROAM_CUDA(cudaMemcpy(c->bits.p, bits, n_words * sizeof(uint32_t),
@@ -896,20 +895,18 @@ roam_status roam_load_grid(roam_ctx *c, const roam_grid_desc *desc, const uint32
     ROAM_TRY(ensure(c->brick_t0, n_bricks));
     ROAM_TRY(ensure(c->brick_t1, n_bricks));
     g.bits = c->bits.p;
-    g.prefix = c->prefix.p;
     g.cells = c->cells.p;
     g.brick_dist = c->brick_dist.p;
     g.labels = nullptr;
     g.n_fields = 0;
-    launch_grid_prefix(c->bits.p, c->prefix.p, c->block_sums.p, c->cells.p, n_words, 0);
+    launch_grid_cells(c->bits.p, c->cells.p, c->block_sums.p, n_words, 0);
     ROAM_TRY(launched("grid prefix"));
     launch_brick_dist(g, c->brick_occ.p, c->brick_t0.p, c->brick_t1.p, c->brick_dist.p, 0);
     ROAM_TRY(launched("brick distance map"));
-    uint32_t last_pre = 0, last_word = 0;
-    ROAM_CUDA(cudaMemcpy(&last_pre, c->prefix.p + n_words - 1, 4, cudaMemcpyDeviceToHost));
-    ROAM_CUDA(cudaMemcpy(&last_word, c->bits.p + n_words - 1, 4, cudaMemcpyDeviceToHost));
+    uint2 last{};
+    ROAM_CUDA(cudaMemcpy(&last, c->cells.p + n_words - 1, sizeof(last), cudaMemcpyDeviceToHost));
     c->n_words = n_words;
-    c->n_occ = (int64_t)last_pre + __builtin_popcount(last_word);
+    c->n_occ = (int64_t)last.y + __builtin_popcount(last.x);
     c->gd = *desc;
     c->has_grid = true;
     return ROAM_OK;
@@ -1250,7 +1247,7 @@ roam_status roam_assign_fields(roam_ctx *c, int n_fields, uint16_t *labels, int3
     cudaStream_t s = (cudaStream_t)stream;
     ROAM_TRY(ensure(c->assign_vox, (size_t)S));
     ROAM_TRY(ensure(c->assign_scratch, assign_scratch_bytes((uint32_t)S, (int64_t)c->g.bx * c->g.by * c->g.bz)));
-    launch_assign(c->bits.p, c->prefix.p, c->n_words, c->g.gx, c->g.gy, c->g.gz, (uint32_t)S, n_fields, c->assign_vox.p,
+    launch_assign(c->cells.p, c->n_words, c->g.gx, c->g.gy, c->g.gz, (uint32_t)S, n_fields, c->assign_vox.p,
                   labels, boxes, c->assign_scratch.p, c->n_sm, s);
     ROAM_TRY(launched("field assignment"));
     ROAM_CUDA(cudaStreamSynchronize(s));
