@@ -502,20 +502,15 @@ __host__ __device__ constexpr int64_t ts_off(int a)
 // API layout -> every layer transposed ([K][N]) then its bias [N]
 __global__ void k_teacher_pack_simt(const float *__restrict__ w, float *__restrict__ wt)
 {
-    for (int a = 0; a < kTLayers; ++a) {
-        const int N = t_out(a), K = t_in(a);
-        const float *src = w + t_off(a);
-        float *dst = wt + ts_off(a);
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)N * K + N;
-             e += (int64_t)gridDim.x * blockDim.x) {
-            if (e < (int64_t)N * K) {
-                const int k = (int)(e / N), nn = (int)(e % N);
-                dst[e] = src[(int64_t)nn * K + k];
-            } else {
-                dst[e] = src[e];
-            }
-        }
-    }
+    const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    auto layer = [&](auto AA) {
+        constexpr int a = decltype(AA)::value, N = t_out(a), K = t_in(a);
+        constexpr int64_t from = t_off(a), to = ts_off(a);
+        for (int e = first; e < N * K + N; e += stride)
+            wt[to + e] = w[from + (e < N * K ? (e % N) * K + e / N : e)];
+    };
+    layer(Int<0>{}); layer(Int<1>{}); layer(Int<2>{}); layer(Int<3>{}); layer(Int<4>{}); layer(Int<5>{});
+    layer(Int<6>{}); layer(Int<7>{}); layer(Int<8>{}); layer(Int<9>{}); layer(Int<10>{}); layer(Int<11>{});
 }
 
 // the matrix layers of one tile in order: layers 1-8, the feature head, layer 10
@@ -542,7 +537,7 @@ __global__ void __launch_bounds__(256, 1) k_teacher_simt(const float *__restrict
     float *red = ring + kSStages * kSStage;                // [256] partial sums
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int sg = lane & 7, og = lane >> 3;
-    const int smp = tid % S, part = tid / S;
+    const int smp = tid % S, part = tid / S;               // (part >= NP: no point, at S = 96)
     __shared__ int4 lay[10];                               // offset, inputs, outputs, bias offset
     if (tid < 10) {
         const int a = ts_layer(tid), o = (int)ts_off(a), K = t_in(a), N = t_out(a);
@@ -599,8 +594,8 @@ __global__ void __launch_bounds__(256, 1) k_teacher_simt(const float *__restrict
         }
         auto rows = [&](auto HALF, int r0, int nr) {
             constexpr bool kHalf = decltype(HALF)::value != 0;
-            constexpr int ng = kHalf ? (G > 1 ? G / 2 : 1) : G;
-            const int g0 = kHalf && G > 1 ? (warp >> 2) * ng : 0;
+            constexpr int ng = kHalf ? (G + 1) / 2 : G;
+            const int g0 = kHalf ? (warp >> 2) * ng : 0;
             const float *wr = ring + slot * kSStage + col;
             const float *xr = X + (int64_t)(base + r0) * XS + 4 * (sg + 8 * g0);
 #pragma unroll 4
@@ -611,6 +606,7 @@ __global__ void __launch_bounds__(256, 1) k_teacher_simt(const float *__restrict
                                       make_float2(w1.z, w1.w)};
 #pragma unroll
                 for (int g = 0; g < ng; ++g) {
+                    if (kHalf && g0 + g >= G) continue;
                     const float4 x4 = *reinterpret_cast<const float4 *>(xr + k * XS + 32 * g);
                     const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
 #pragma unroll
@@ -629,17 +625,17 @@ __global__ void __launch_bounds__(256, 1) k_teacher_simt(const float *__restrict
             feed();
             const int nr = min(kSRows, K - r0);
             if (!half) rows(Int<0>{}, r0, nr);
-            else if (G > 1 || warp < 4) rows(Int<1>{}, r0, nr);
+            else rows(Int<1>{}, r0, nr);
             if (++slot == kSStages) slot = 0;
         }
         __syncthreads();                                   // every thread has read the input
-        const int ng = half ? (G > 1 ? G / 2 : (warp < 4 ? 1 : 0)) : G;
-        const int g0 = half && G > 1 ? (warp >> 2) * ng : 0;
+        const int ng = half ? (G + 1) / 2 : G;
+        const int g0 = half ? (warp >> 2) * ng : 0;
 #pragma unroll
         for (int j = 0; j < 8; ++j)
 #pragma unroll
             for (int g = 0; g < G; ++g) {
-                if (g >= ng) continue;
+                if (g >= ng || g0 + g >= G) continue;
                 float v[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -656,7 +652,7 @@ __global__ void __launch_bounds__(256, 1) k_teacher_simt(const float *__restrict
         float *col = X + (int64_t)kTW * XS + smp;
         if (part == 0)
             for (int a = 0; a < 3; ++a) col[a * XS] = x[a];
-        for (int k = part; k < L; k += NP)
+        for (int k = part; k < (part < NP ? L : 0); k += NP)
             for (int a = 0; a < 3; ++a) {
                 float s, c;
                 sincospif(x[a] * (float)(1 << k), &s, &c);
@@ -684,8 +680,9 @@ __global__ void __launch_bounds__(256, 1) k_teacher_simt(const float *__restrict
         {
             const float *Wd = wt + ts_off(8);
             float s = 0.f;
+            const int k1 = part < NP ? (part + 1) * (kTW / NP) : 0;
 #pragma unroll 8
-            for (int k = part * (kTW / NP); k < (part + 1) * (kTW / NP); ++k) s = fmaf(X[(int64_t)k * XS + smp], __ldg(Wd + k), s);
+            for (int k = part * (kTW / NP); k < k1; ++k) s = fmaf(X[(int64_t)k * XS + smp], __ldg(Wd + k), s);
             red[tid] = s;
         }
         __syncthreads();
@@ -749,13 +746,22 @@ void launch_teacher_simt(const float *wt, TeacherAffine aff, int64_t n, const fl
                          int n_sm, cudaStream_t s)
 {
     if (n <= 0) return;
-    // one tile per block at a time: the tile size whose waves end first, from
-    // the measured time of one tile of 128 / 64 / 32 points (424 / 248 / 164 us)
-    auto waves = [&](int S) { return (double)(((n + S - 1) / S + n_sm - 1) / n_sm); };
-    const double c16 = 424 * waves(128), c8 = 248 * waves(64), c4 = 164 * waves(32);
-    if (c16 <= c8 && c16 <= c4) launch_simt_t<16>(wt, aff, n, p, d, out, n_sm, s);
-    else if (c8 <= c4) launch_simt_t<8>(wt, aff, n, p, d, out, n_sm, s);
-    else launch_simt_t<4>(wt, aff, n, p, d, out, n_sm, s);
+    // One tile per block at a time.  Whole waves of 128-point tiles first, then
+    // the rest in the tile size whose waves end first, from the measured time of
+    // one tile of 128 / 96 / 64 / 32 points (424 / 330 / 248 / 164 us)
+    const int64_t wave = (int64_t)128 * n_sm, n0 = n / wave * wave, r = n - n0;
+    if (n0 > 0) launch_simt_t<16>(wt, aff, n0, p, d, out, n_sm, s);
+    if (r == 0) return;
+    auto waves = [&](int S) { return (double)(((r + S - 1) / S + n_sm - 1) / n_sm); };
+    const double c16 = 424 * waves(128), c12 = 330 * waves(96), c8 = 248 * waves(64), c4 = 164 * waves(32);
+    const double best = c16 < c12 ? (c16 < c8 ? c16 : c8) : (c12 < c8 ? c12 : c8);
+    p += 3 * n0;
+    d += 3 * n0;
+    out += n0;
+    if (c4 <= best) launch_simt_t<4>(wt, aff, r, p, d, out, n_sm, s);
+    else if (c8 <= best) launch_simt_t<8>(wt, aff, r, p, d, out, n_sm, s);
+    else if (c12 <= best) launch_simt_t<12>(wt, aff, r, p, d, out, n_sm, s);
+    else launch_simt_t<16>(wt, aff, r, p, d, out, n_sm, s);
 }
 
 }  // namespace roam

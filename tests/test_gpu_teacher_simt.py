@@ -1,5 +1,5 @@
-"""The FP32 teacher over its tile sizes (32, 64 and 128 points, chosen by the
-number of points) and their remainders, against the oracle at the first and
+"""The FP32 teacher over its tile sizes (32, 64, 96 and 128 points, chosen by
+the number of points; whole waves, then a rest) and their remainders, against the oracle at the first and
 last points and a sample of the others; the bar of the FP32 teacher's other
 test (1e-4: FP32 sums of up to 319 terms over 11 layers)."""
 import numpy as np
@@ -21,7 +21,7 @@ def roam():
     return roam
 
 
-@pytest.mark.parametrize("n", [1, 31, 33, 4864, 9727, 9800, 15999, 20011, 40001])
+@pytest.mark.parametrize("n", [1, 31, 33, 4864, 9727, 9800, 14001, 15999, 20011, 32768, 40001])
 def test_teacher_f32_tiles(roam, room32, n):
     r = roam.Roam(0)
     w, aff = F.teacher_weights(7, bias_scale=0.1), F.scene_affine(room32.scene)
