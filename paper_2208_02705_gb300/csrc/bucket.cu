@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(1024) k_scan(uint32_t *hist, int n_fields, int
 {
     __shared__ uint32_t warp_a[32], warp_b[32];
     extern __shared__ uint32_t tile_off[];   // [n_fields + 1]
+    pdl_begin();
     const int per = (n_fields + blockDim.x - 1) / blockDim.x;
     const int f0 = threadIdx.x * per;
     uint32_t cs = 0, ts = 0, hit = 0;
@@ -257,6 +258,7 @@ __global__ void __launch_bounds__(512) k_scatter_blk(const uint32_t *cnt, const 
     extern __shared__ uint32_t sh[];
     uint32_t *cnt_s = sh, *base_s = sh + n_fields;
     for (int f = threadIdx.x; f < n_fields; f += blockDim.x) cnt_s[f] = 0u;
+    pdl_begin();
     __syncthreads();
     SlotIter it{cnt, recs, live_count ? *live_count : n_fixed, (uint32_t)R};
     const uint64_t tot = keys16 ? (uint64_t)n_fixed : it.total();
@@ -304,13 +306,11 @@ void scan_and_scatter(const uint32_t *cnt, const uint32_t *recs, const uint32_t 
                       int grid, cudaStream_t s, ClassBounds cb)
 {
     const bool blk = b.tile_off != nullptr && n_fields <= kMaxFieldsBlk;
-    k_scan<<<1, 1024, (size_t)(n_fields + 1) * sizeof(uint32_t), s>>>(b.hist, n_fields, tile, group < 1 ? 1 : group,
-                                                                       b.offsets, b.cursor, b.tiles,
-                                                                       blk ? b.tile_off : nullptr, ctr, cb);
+    launch_pdl(k_scan, 1, 1024, (size_t)(n_fields + 1) * sizeof(uint32_t), s, b.hist, n_fields, tile,
+               group < 1 ? 1 : group, b.offsets, b.cursor, b.tiles, blk ? b.tile_off : nullptr, ctr, cb);
     if (blk)
-        k_scatter_blk<<<grid, 512, 2 * (size_t)n_fields * sizeof(uint32_t), s>>>(
-            cnt, recs, live_count, n_fixed, R, keys16, n_fields, b.cursor, b.sorted, b.tile_off, b.offsets, b.tiles,
-            tile, ctr);
+        launch_pdl(k_scatter_blk, grid, 512, 2 * (size_t)n_fields * sizeof(uint32_t), s, cnt, recs, live_count, n_fixed,
+                   R, keys16, n_fields, b.cursor, b.sorted, b.tile_off, b.offsets, b.tiles, tile, ctr);
     else
         k_scatter<<<grid, 512, 0, s>>>(cnt, recs, live_count, n_fixed, R, keys16, n_fields, b.cursor, b.sorted);
 }

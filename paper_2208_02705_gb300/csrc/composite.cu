@@ -38,6 +38,7 @@ __device__ __forceinline__ void step(float4 v, float t, float delta, float &T, f
 __global__ void __launch_bounds__(256) k_composite_round(RoundArgs a)
 {
     const MarchParams &p = a.mp;
+    pdl_begin();
     const uint32_t n_live = p.live_count ? *p.live_count : p.n_rays;
     const uint32_t n_pad = (n_live + 31u) & ~31u;
     const uint32_t stride = gridDim.x * blockDim.x;
@@ -198,7 +199,7 @@ void launch_composite_round(const MarchParams &mp, const float4 *sr, uint32_t *n
                             cudaStream_t s)
 {
     RoundArgs a{mp, sr, next_live, next_count, t_stop, bg[0], bg[1], bg[2], rgb, depth, opacity};
-    k_composite_round<<<grid, 256, 0, s>>>(a);
+    launch_pdl(k_composite_round, grid, 256, 0, s, a);
 }
 
 void launch_composite_flat(int64_t n_rays, int n_max, const uint32_t *count, const float4 *sr, const float *t,

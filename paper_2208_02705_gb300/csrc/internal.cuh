@@ -25,6 +25,34 @@ inline void raise_smem_limit(const void *kernel, int bytes, int (&cached)[kMaxDe
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess && tracked)
         cached[dev] = bytes;
 }
+
+// Programmatic dependent launch: kernels of one call follow one another closely
+// (a render round is five launches of a few microseconds each), so a kernel is
+// launched while its predecessor ends and starts with pdl_begin, which waits for
+// all of the predecessor's work and then lets its own successor be launched.
+// Nothing global is touched before it.  (After a launch of another kind, and
+// in a launch without the attribute, the order is the stream's.)
+__device__ __forceinline__ void pdl_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);      // (an error stays for the launch check)
+}
+
 constexpr int kBrickShift = 3;    // 8^3-voxel bricks for empty-space skipping
 constexpr int kMaxViews = 256;
 

@@ -309,6 +309,7 @@ __device__ __forceinline__ float empty_jump(int dd, int ix, int iy, int iz, cons
 __global__ void __launch_bounds__(256) k_march(GridDev g, MarchParams p)
 {
     extern __shared__ uint32_t s_hist[];      // per-block field histogram (when p.hist)
+    pdl_begin();
     const uint32_t n_live = p.live_count ? *p.live_count : p.n_rays;
     if (blockIdx.x == 0 && threadIdx.x == 0 && p.live_count != nullptr) {
         // the count slot the composite of this round fills is the one the
@@ -446,7 +447,7 @@ void launch_brick_dist(GridDev g, uint8_t *occ, uint16_t *t0, uint16_t *t1, uint
 
 void launch_march(const GridDev &g, const MarchParams &p, int grid, cudaStream_t s)
 {
-    k_march<<<grid, 256, p.hist ? (size_t)g.n_fields * sizeof(uint32_t) : 0, s>>>(g, p);
+    launch_pdl(k_march, grid, 256, p.hist ? (size_t)g.n_fields * sizeof(uint32_t) : 0, s, g, p);
 }
 
 }  // namespace roam

@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(kThreads, SimtShape<W, H>::kBlocks)
         entries[e] = en;
     }
     __syncthreads();
+    pdl_begin();
 
     // tiles of the width class split evenly over the blocks, in order
     const uint32_t c0 = ctr->class_tiles[w.cls], n_tiles = ctr->class_tiles[w.cls + 1] - c0;
@@ -273,7 +274,7 @@ static void launch_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs
     static int smem_set[kMaxDevices] = {};
     raise_smem_limit((const void *)k_mlp_simt<W, H>, (int)F::kSmem, smem_set);
     // one wave of resident blocks; each takes a contiguous run of tiles
-    k_mlp_simt<W, H><<<n_sm * F::kBlocks, kThreads, F::kSmem, s>>>(w, src, b, ctr, out);
+    launch_pdl(k_mlp_simt<W, H>, n_sm * F::kBlocks, kThreads, F::kSmem, s, w, src, b, ctr, out);
 }
 
 void launch_mlp_simt(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out,

@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * TcShape<W, H, F8>:
     const uint32_t imga = smem_u32(IMG);
     const float *tab = reinterpret_cast<const float *>(IMG + S::kMatBytes + S::kOutBytes);
 
+    pdl_begin();
     // this width class's tiles (a multiple of kSlots apart: bucket padding)
     const Tile *tiles = b.tiles + ctr->class_tiles[cls];
     const uint32_t n_groups = (ctr->class_tiles[cls + 1] - ctr->class_tiles[cls]) / kSlots;
@@ -525,9 +526,8 @@ void launch_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Co
     raise_smem_limit((const void *)k_mlp_tc<W, H, F8>, smem, smem_set);
     const void *img = F8 ? w.wimg8 : w.wimg;
     const int64_t ib = F8 ? w.img8_bytes : w.img_bytes;
-    k_mlp_tc<W, H, F8><<<n_sm, kSlots * TcShape<W, H, F8>::kSlotThreads, smem, s>>>(img, ib, w.field_base, w.cls, w.affine, w.sigma_scale, w.act,
-                                                        src, b, ctr, out, w.wait_ns ? w.wait_ns : kWaitNs,
-                                                        w.withhold_image);
+    launch_pdl(k_mlp_tc<W, H, F8>, n_sm, kSlots * TcShape<W, H, F8>::kSlotThreads, smem, s, img, ib, w.field_base, w.cls,
+               w.affine, w.sigma_scale, w.act, src, b, ctr, out, w.wait_ns ? w.wait_ns : kWaitNs, w.withhold_image);
 }
 
 #define ROAM_TC_CASES                                                                                   \
