@@ -16,10 +16,11 @@
 // voxels, bounds the distance of the last voxel wanted; only bricks that reach
 // below that bound are candidates; a histogram of their voxels' squared
 // distances narrows the last voxel's key to one bin, and that bin's keys are
-// ranked directly.  Histograms are exchanged through distributed shared
-// memory, so a network costs four cluster barriers and a few L2 latencies, and
-// touches about as many voxels as it takes (instead of every unassigned voxel
-// five times in five launches).
+// ranked directly.  The candidates' keys stay in registers between these steps
+// (up to four per thread), histograms are pushed into every block's copy
+// through distributed shared memory, so a network costs four cluster barriers
+// and a few L2 latencies, and touches about as many voxels as it takes (instead
+// of every unassigned voxel five times in five launches).
 //
 // The general form, for larger networks: per network
 //   k_hist_select  per digit of the 47-bit key (squared distance << 27 |
@@ -284,7 +285,8 @@ constexpr int kCluster = 8;
 constexpr int kAT = 1024;                   // threads per block
 constexpr int kABins = 1024;                // one per thread
 constexpr int kListMax = 1024;              // keys ranked directly
-constexpr int kCandMax = 7168;              // candidate bricks of one block kept in shared memory
+constexpr int kCandMax = 1536;              // candidate bricks of one block kept in shared memory
+constexpr int kVox = 4;                     // ... and voxels per thread kept in registers
 
 struct BrickLists {
     uint32_t *n;           // [2]: bricks with voxels, voxels
@@ -378,35 +380,40 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
                     int n, uint32_t per)
 {
     cg::cluster_group cluster = cg::this_cluster();
-    __shared__ uint32_t hist_a[kABins], hist_b[kABins], scratch[32];
+    // a block's own histogram, and the cluster's sum of one (every block's copy)
+    __shared__ uint32_t hist[kABins], sum[2][kABins], scratch[32];
     __shared__ unsigned long long list[kListMax];         // block 0's is the cluster's
-    __shared__ uint32_t list_n, sel_bin, sel_before, sel_count, anchor_s, cand_n;
-    __shared__ unsigned long long thr_s;
-    __shared__ uint32_t cand[kCandMax];
+    __shared__ uint32_t list_n, sel_bin, sel_before, sel_count;
+    __shared__ unsigned long long thr_s, anchor_s, cand_s;
+    // candidate bricks, and where each one's voxels start among the candidates'
+    __shared__ uint32_t cand[kCandMax], cand_at[kCandMax], cand_kept[kCandMax];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster.block_rank(), n_bricks = L.n[0];
 
-    hist_a[tid] = 0u;
-    hist_b[tid] = 0u;
+    hist[tid] = sum[0][tid] = sum[1][tid] = 0u;
     if (tid == 0) {
         list_n = 0u;
-        cand_n = 0u;
+        cand_s = 0ull;
     }
     cluster.sync();
-    // the cluster's sum of a histogram, this thread's bin
-    auto reduce = [&](uint32_t *h) {
-        uint32_t v[kCluster], sum = 0;
+    // adds the block's histogram to every block's copy of the cluster's sum h
+    // (a push: after the cluster's barrier nothing is read across blocks), and clears it
+    auto share = [&](uint32_t *h) {
+        __syncthreads();
+        const uint32_t v = hist[tid];
+        if (v) {
 #pragma unroll
-        for (int q = 0; q < kCluster; ++q) v[q] = cluster.map_shared_rank(h, q)[tid];
-#pragma unroll
-        for (int q = 0; q < kCluster; ++q) sum += v[q];
-        return sum;
+            for (int q = 0; q < kCluster; ++q) atomicAdd(&cluster.map_shared_rank(h, q)[tid], v);
+            hist[tid] = 0u;
+        }
+        cluster.sync();
     };
-    // the bin that holds item `want` (0-based) of the summed histogram; every
-    // block finds the same.  False: fewer items.
+    // the bin that holds item `want` (0-based) of the summed histogram, which is
+    // cleared; every block finds the same.  False: fewer items.
     auto select = [&](uint32_t *h, uint32_t want) -> bool {
         if (tid == 0) sel_bin = 0xffffffffu;
-        const uint32_t c = reduce(h), incl = block_scan(c, scratch);
+        const uint32_t c = h[tid], incl = block_scan(c, scratch);
+        h[tid] = 0u;
         if (want >= incl - c && want < incl) {
             sel_bin = (uint32_t)tid;
             sel_before = incl - c;
@@ -419,24 +426,24 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
     uint32_t cursor = 0;
     for (int net = 0; net + 1 < n; ++net) {
         // ---- anchor: the first unassigned rank from the cursor (every block looks) ----
-        uint32_t base = cursor;
-        for (;; base += kAT) {
-            if (tid == 0) anchor_s = 0xffffffffu;
+        for (uint32_t base = cursor;; base += kAT) {
+            if (tid == 0) anchor_s = ~0ull;
             __syncthreads();
             const uint32_t i = base + (uint32_t)tid;
+            const uint32_t v = i < S ? __ldg(&vox[i]) : 0u;
             const unsigned m = __ballot_sync(0xffffffffu, i < S && __ldcg(&field[i]) == kFree);
-            if (lane == 0 && m) atomicMin(&anchor_s, base + (uint32_t)(warp * 32 + __ffs(m) - 1));
+            if (m && lane == __ffs(m) - 1) atomicMin(&anchor_s, (unsigned long long)i << 32 | v);
             __syncthreads();
-            if (anchor_s != 0xffffffffu || base + kAT >= S) break;
+            if (anchor_s != ~0ull || base + kAT >= S) break;
             __syncthreads();
         }
-        const uint32_t anchor = anchor_s;
-        if (anchor == 0xffffffffu) {                        // (the same in every block)
+        const unsigned long long found = anchor_s;
+        if (found == ~0ull) {                               // (the same in every block)
             if (rank == 0 && tid == 0) st->status = 1u;
             break;
         }
-        cursor = anchor;
-        const uint32_t av = __ldg(&vox[anchor]);
+        cursor = (uint32_t)(found >> 32);
+        const uint32_t av = (uint32_t)found;
         const int ax = (int)(av % (uint32_t)gx), ay = (int)((av / (uint32_t)gx) % (uint32_t)gy),
                   az = (int)(av / ((uint32_t)gx * (uint32_t)gy));
         // smallest and largest squared distance of a brick's voxels to the anchor
@@ -459,10 +466,10 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
             if (!c) continue;
             uint32_t lo, hi;
             reach(L.coord[b], lo, hi);
-            atomicAdd(&hist_a[dist_bin(hi)], c);
+            atomicAdd(&hist[dist_bin(hi)], c);
         }
-        cluster.sync();
-        const bool enough = select(hist_a, per - 1u);
+        share(sum[0]);
+        const bool enough = select(sum[0], per - 1u);
         if (!enough) {                                      // fewer voxels than asked for
             if (rank == 0 && tid == 0) st->status = 1u;
             break;
@@ -480,16 +487,48 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
             uint32_t lo, hi;
             reach(L.coord[b], lo, hi);
             if (lo >= bound) continue;
-            const uint32_t q = atomicAdd(&cand_n, 1u);
-            if (q < (uint32_t)kCandMax) cand[q] = b;
+            // its place in the table and its voxels' places, both in one counter
+            const unsigned long long at = atomicAdd(&cand_s, 1ull << 32 | L.count[b]);
+            const uint32_t q = (uint32_t)(at >> 32);
+            if (q < (uint32_t)kCandMax) {
+                cand[q] = b;
+                cand_at[q] = (uint32_t)at;
+                cand_kept[q] = 0u;
+            }
         }
         __syncthreads();
-        // (past the table a warp goes over all of its block's bricks)
-        const uint32_t nc = cand_n;
+        const uint32_t nc = (uint32_t)(cand_s >> 32), nv = (uint32_t)cand_s;
         const bool table = nc <= (uint32_t)kCandMax;
+        // a few voxels per thread: their keys stay in registers
+        const bool few = table && nv <= kVox * (uint32_t)kAT;
+        unsigned long long vk[kVox];
+        uint32_t vq[kVox];
+        uint16_t vl[kVox];
+        if (few) {
+#pragma unroll
+            for (int u = 0; u < kVox; ++u) {
+                const uint32_t e = (uint32_t)(u * kAT + tid);
+                vk[u] = ~0ull;
+                if (e >= nv) continue;
+                uint32_t q0 = 0, q1 = nc;                    // the last candidate at or before e
+                while (q1 - q0 > 1) {
+                    const uint32_t mid = (q0 + q1) / 2;
+                    if (cand_at[mid] <= e) q0 = mid; else q1 = mid;
+                }
+                const uint32_t b = cand[q0], c = L.coord[b], at = L.start[b] + (e - cand_at[q0]);
+                const uint32_t l = L.loc[at], r = L.rank[at];
+                const int dx = (int)(c & 255u) * 8 - ax + (int)(l & 7u), dy = (int)((c >> 8) & 255u) * 8 - ay + (int)((l >> 3) & 7u),
+                          dz = (int)((c >> 16) & 255u) * 8 - az + (int)(l >> 6);
+                vk[u] = (unsigned long long)(uint32_t)(dx * dx + dy * dy + dz * dz) << kRankBits | r;
+                vq[u] = q0;
+                vl[u] = (uint16_t)l;
+            }
+        }
+        // else a warp goes over its block's candidates (past the table: over all
+        // of its block's bricks)
         const uint32_t n_own = n_bricks > rank ? (n_bricks - rank + kCluster - 1) / kCluster : 0u;
         const uint32_t n_it = table ? nc : n_own;
-        // every candidate voxel of this warp's bricks: f(entry, key)
+        // every candidate voxel of this warp's bricks: f(brick, voxels, first entry, key of an entry)
         auto visit = [&](auto f) {
             for (uint32_t q = (uint32_t)warp; q < n_it; q += kAT / 32) {
                 const uint32_t b = table ? cand[q] : rank + q * kCluster;
@@ -508,16 +547,24 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
                 });
             }
         };
-        visit([&](uint32_t, uint32_t cnt, uint32_t s0, auto key) {
-            for (uint32_t e = (uint32_t)lane; e < cnt; e += 32) {
-                const unsigned long long k = key(s0 + e);
-                if (k < bound_key) atomicAdd(&hist_b[(uint32_t)(k >> (kRankBits + sh))], 1u);
+        auto each_key = [&](auto f) {
+            if (few) {
+#pragma unroll
+                for (int u = 0; u < kVox; ++u)
+                    if (vk[u] < bound_key) f(vk[u]);
+            } else {
+                visit([&](uint32_t, uint32_t cnt, uint32_t s0, auto key) {
+                    for (uint32_t e = (uint32_t)lane; e < cnt; e += 32) {
+                        const unsigned long long k = key(s0 + e);
+                        if (k < bound_key) f(k);
+                    }
+                });
             }
-        });
-        cluster.sync();
-        hist_a[tid] = 0u;                                   // (every block is past its reads of hist_a)
+        };
+        each_key([&](unsigned long long k) { atomicAdd(&hist[(uint32_t)(k >> (kRankBits + sh))], 1u); });
+        share(sum[1]);
         uint32_t want = per - 1u;
-        select(hist_b, want);
+        select(sum[1], want);
         want -= sel_before;
         // the wanted key lies in [lo_key, lo_key + 2^shift)
         int shift = sh + kRankBits;
@@ -525,19 +572,13 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
         uint32_t left = sel_count;
         // ---- narrow until the bin's keys can be ranked directly (rarely needed) ----
         while (left > (uint32_t)kListMax) {
-            cluster.sync();                                 // every block has read hist_b
-            hist_b[tid] = 0u;
-            __syncthreads();
+            cluster.sync();                                 // every block has read and cleared its sum
             const int ns = max(0, shift - 10);
-            visit([&](uint32_t, uint32_t cnt, uint32_t s0, auto key) {
-                for (uint32_t e = (uint32_t)lane; e < cnt; e += 32) {
-                    const unsigned long long k = key(s0 + e);
-                    if (k >= lo_key && k < bound_key && (k - lo_key) >> shift == 0ull)
-                        atomicAdd(&hist_b[(uint32_t)((k - lo_key) >> ns)], 1u);
-                }
+            each_key([&](unsigned long long k) {
+                if (k >= lo_key && (k - lo_key) >> shift == 0ull) atomicAdd(&hist[(uint32_t)((k - lo_key) >> ns)], 1u);
             });
-            cluster.sync();
-            select(hist_b, want);
+            share(sum[1]);
+            select(sum[1], want);
             want -= sel_before;
             lo_key += (unsigned long long)sel_bin << ns;
             shift = ns;
@@ -548,18 +589,14 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
         {
             uint32_t *ln = cluster.map_shared_rank(&list_n, 0);
             unsigned long long *lp = cluster.map_shared_rank(list, 0);
-            visit([&](uint32_t, uint32_t cnt, uint32_t s0, auto key) {
-                for (uint32_t e = (uint32_t)lane; e < cnt; e += 32) {
-                    const unsigned long long k = key(s0 + e);
-                    if (k >= lo_key && k < bound_key && (k - lo_key) >> shift == 0ull) {
-                        const uint32_t at = atomicAdd(ln, 1u);
-                        if (at < (uint32_t)kListMax) lp[at] = k;
-                    }
+            each_key([&](unsigned long long k) {
+                if (k >= lo_key && (k - lo_key) >> shift == 0ull) {
+                    const uint32_t at = atomicAdd(ln, 1u);
+                    if (at < (uint32_t)kListMax) lp[at] = k;
                 }
             });
         }
         cluster.sync();
-        hist_b[tid] = 0u;                                   // (every block is past its reads of hist_b)
         if (rank != 0 && (uint32_t)tid < left) list[tid] = cluster.map_shared_rank(list, 0)[tid];
         __syncthreads();
         if ((uint32_t)tid < left) {
@@ -572,29 +609,47 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
         __syncthreads();
         const unsigned long long thr = thr_s;
         // ---- take: keys up to the threshold join the network; each brick's list closes up ----
-        visit([&](uint32_t b, uint32_t cnt, uint32_t s0, auto key) {
-            uint32_t kept = 0;
-            for (uint32_t e0 = 0; e0 < cnt; e0 += 32) {
-                const uint32_t e = s0 + e0 + (uint32_t)lane;
-                const bool in = e0 + (uint32_t)lane < cnt;
-                const uint32_t r = in ? L.rank[e] : 0u;
-                const uint16_t l = in ? L.loc[e] : (uint16_t)0;
-                const bool take = in && key(in ? e : s0) <= thr;
-                const unsigned km = __ballot_sync(0xffffffffu, in && !take);
-                if (take) __stcg(&field[r], (uint16_t)net);
-                __syncwarp();
-                if (in && !take) {
-                    const uint32_t at = s0 + kept + (uint32_t)__popc(km & ((1u << lane) - 1u));
+        if (few) {
+            // (every entry was read above: the kept ones close up in any order)
+#pragma unroll
+            for (int u = 0; u < kVox; ++u) {
+                if (vk[u] == ~0ull) continue;
+                const uint32_t r = (uint32_t)vk[u] & ((1u << kRankBits) - 1u);
+                if (vk[u] <= thr) {
+                    __stcg(&field[r], (uint16_t)net);
+                } else {
+                    const uint32_t at = L.start[cand[vq[u]]] + atomicAdd(&cand_kept[vq[u]], 1u);
                     L.rank[at] = r;
-                    L.loc[at] = l;
+                    L.loc[at] = vl[u];
                 }
-                __syncwarp();
-                kept += (uint32_t)__popc(km);
             }
-            if (lane == 0) L.count[b] = kept;
-        });
+            __syncthreads();
+            for (uint32_t q = (uint32_t)tid; q < nc; q += kAT) L.count[cand[q]] = cand_kept[q];
+        } else {
+            visit([&](uint32_t b, uint32_t cnt, uint32_t s0, auto key) {
+                uint32_t kept = 0;
+                for (uint32_t e0 = 0; e0 < cnt; e0 += 32) {
+                    const uint32_t e = s0 + e0 + (uint32_t)lane;
+                    const bool in = e0 + (uint32_t)lane < cnt;
+                    const uint32_t r = in ? L.rank[e] : 0u;
+                    const uint16_t l = in ? L.loc[e] : (uint16_t)0;
+                    const bool take = in && key(in ? e : s0) <= thr;
+                    const unsigned km = __ballot_sync(0xffffffffu, in && !take);
+                    if (take) __stcg(&field[r], (uint16_t)net);
+                    __syncwarp();
+                    if (in && !take) {
+                        const uint32_t at = s0 + kept + (uint32_t)__popc(km & ((1u << lane) - 1u));
+                        L.rank[at] = r;
+                        L.loc[at] = l;
+                    }
+                    __syncwarp();
+                    kept += (uint32_t)__popc(km);
+                }
+                if (lane == 0) L.count[b] = kept;
+            });
+        }
         __syncthreads();
-        if (tid == 0) cand_n = 0u;
+        if (tid == 0) cand_s = 0ull;
         cluster.sync();                                     // the labels and lists are in place; block 0's list is read
         if (rank == 0 && tid == 0) list_n = 0u;
     }
@@ -604,8 +659,8 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
 }  // namespace
 
 // Networks up to this many voxels are built from the brick lists.  Measured per
-// network (GB300): 16 us against 52 us for the general form at 2,000 voxels,
-// 49 us at 33,000, where the general form takes 155; from 65,000 on, 8 blocks
+// network (GB300): 11 us against 52 us for the general form at 2,000 voxels,
+// 56 us at 33,000, where the general form takes 155; from 65,000 on, 8 blocks
 // against the whole chip, the two meet (89 us general at 67,000).
 constexpr uint32_t kBrickMaxPer = 65536u;
 
