@@ -29,8 +29,14 @@
 // as many steps to FP64.  What a ray's set-up shares with its view is formed
 // once per view (k_occ_views): the FP64 sines and cosines of the pixel columns
 // and rows, the first plane index per axis and direction, and the camera's
-// voxel.  Measured (GB300, four 1024x512 scans of a 256^3 floor): rays 3550 ->
-// 1335 us, voxel passes 225 -> 65 us.
+// voxel.  Beside that, the walk waits for the word bits it checks: looking at
+// them one word later, blocks of 128 (which end sooner than 256 where the
+// rays' lengths differ): 1318 -> 1071 us.  A step in FP64 takes one reciprocal per
+// axis (Newton steps, no division) and forms the end's parameter only where it
+// can be the next event: 1045.  Eight blocks per SM at 64 registers, some values
+// spilled: 931 (seven at 72: 973; six at 80, none spilled: 1045).  Measured (GB300, four
+// 1024x512 scans of a 256^3 floor): rays 3550 -> 931 us, voxel passes
+// 225 -> 65 us.
 #include "internal.cuh"
 
 namespace roam {
@@ -82,7 +88,7 @@ __global__ void __launch_bounds__(256) k_occ_views(GridDev g, const DevCamera *c
     }
 }
 
-__global__ void __launch_bounds__(256) k_occ_rays(GridDev g, const DevCamera *cams, int view, const OccView *views,
+__global__ void __launch_bounds__(128, 8) k_occ_rays(GridDev g, const DevCamera *cams, int view, const OccView *views,
                                                   const double2 *tab, const float *depth, const float *opacity,
                                                   float a_min, uint32_t *hit, uint32_t *free_bits, uint32_t *hit_bits)
 {
@@ -118,39 +124,55 @@ __global__ void __launch_bounds__(256) k_occ_rays(GridDev g, const DevCamera *ca
         // per axis: next plane index (exact in FP32), step, crossing parameter
         // and the bound on its FP32 error
         float kf[3], sf[3], inf[3], tf[3], er[3];
-        const float dmax = fmaxf(fmaxf(fabsf((float)dv[0]), fabsf((float)dv[1])), fabsf((float)dv[2]));
+        const float d32[3] = {(float)dv[0], (float)dv[1], (float)dv[2]};
+        const float dmax = fmaxf(fmaxf(fabsf(d32[0]), fabsf(d32[1])), fabsf(d32[2]));
         // (no crossing inside the grid lies past t_grid)
         const float t_grid = reach / dmax;
         const float e_t = 4.7683716e-7f * fminf(fabsf(te), t_grid);      // 2^-21 t
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const float df = (float)dv[a];
-            sf[a] = dv[a] > 0.0 ? 1.f : (dv[a] < 0.0 ? -1.f : 0.f);
-            kf[a] = vw.k0[dv[a] > 0.0 ? 0 : 1][a];
+            const float df = d32[a];
             const bool crosses = fabsf(df) >= 1e-20f;            // (else no plane before the end)
+            sf[a] = crosses ? copysignf(1.f, df) : 0.f;
+            kf[a] = vw.k0[df > 0.f ? 0 : 1][a];
             inf[a] = crosses ? 1.f / df : 0.f;
             er[a] = crosses ? fmaf(1.1920929e-7f, fabsf(gf[a] * inf[a]), e_t) : 0.f;
             tf[a] = crosses ? fmaf(kf[a], vf, gf[a]) * inf[a] : 3.0e38f;
         }
-        auto t64_of = [&](int a, double k) {
-            return ((double)g.origin[a] + k * (double)vf - (double)of[a]) * (1.0 / dv[a]);
+        // 1 / d in FP64, two Newton steps from the FP32 reciprocal (a division is
+        // several times as many FP64 operations, each of which takes its turn)
+        auto inv64 = [&](int a) {
+            double r = (double)inf[a];
+            r = fma(fma(-dv[a], r, 1.0), r, r);
+            return fma(fma(-dv[a], r, 1.0), r, r);
+        };
+        auto t64_of = [&](int a, double k, double inv) {
+            return ((double)g.origin[a] + k * (double)vf - (double)of[a]) * inv;
         };
         // the first interval's voxel: the camera's, unless it lies on a plane
         int cc[3] = {vw.cell[0], vw.cell[1], vw.cell[2]};
         if (vw.on_plane) {
             double t1 = (double)D / (double)A;
             for (int a = 0; a < 3; ++a)
-                if (sf[a] != 0.f) t1 = fmin(t1, t64_of(a, (double)kf[a]));
+                if (sf[a] != 0.f) t1 = fmin(t1, t64_of(a, (double)kf[a], inv64(a)));
             for (int a = 0; a < 3; ++a)
                 cc[a] = (int)floor(((double)of[a] + 0.5 * t1 * dv[a] - (double)g.origin[a]) * (1.0 / (double)vf));
         }
         // free bits of the current 32-voxel word, flushed when the word changes;
         // every ray of a view starts at the camera, so the words near it are
         // hit by all of them: bits already set (they are only ever set during
-        // a scan) skip the atomic
+        // a scan) skip the atomic.  What a word's bits were is read when it is
+        // left and looked at when the next word is left, so the read's latency
+        // passes under the walk (an older value only costs an atomic more)
         uint32_t word = 0xffffffffu, mask = 0u;
+        uint32_t old_word = 0u, old_mask = 0u, old_bits = 0u;
         auto flush = [&]() {
-            if (mask && (__ldcg(&free_bits[word]) & mask) != mask) atomicOr(&free_bits[word], mask);
+            if (old_mask & ~old_bits) atomicOr(&free_bits[old_word], old_mask);
+            old_mask = mask;
+            if (mask) {
+                old_word = word;
+                old_bits = __ldcg(&free_bits[word]);
+            }
         };
         // false once the ray has left the grid for good
         auto mark_if_inside = [&]() -> bool {
@@ -167,6 +189,7 @@ __global__ void __launch_bounds__(256) k_occ_rays(GridDev g, const DevCamera *ca
             mask |= 1u << (cc[0] & 31);
             return true;
         };
+        const float len = sqrtf(d32[0] * d32[0] + d32[1] * d32[1] + d32[2] * d32[2]);
         const float t_min = 1e-8f * vf / dmax;                  // (above the 1e-9 voxel rule)
         float cur_hi = 0.f;                                     // the last crossing's parameter and its error bound
         for (int guard = 0; guard < 3 * 65536; ++guard) {
@@ -199,20 +222,26 @@ __global__ void __launch_bounds__(256) k_occ_rays(GridDev g, const DevCamera *ca
             }
             // FP64: the parameter of the last plane crossed (0 before any)
             // and every axis' next crossing, as the definition computes them
-            const double t_end = (double)D / (double)A;
+            // (the end only where it may be the next event)
+            const double t_end = te - e_t <= m1 + e1 || !(te >= 0.f) ? (double)D / (double)A : 1e300;
             double t_cur = 0.0, t_next = t_end;
             double t64[3];
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 t64[q] = 1e300;
                 if (sf[q] == 0.f) continue;
-                const double tp = t64_of(q, (double)kf[q] - (double)sf[q]);
+                const double inv = inv64(q), tp = t64_of(q, (double)(kf[q] - sf[q]), inv);
                 if (tp > t_cur) t_cur = tp;
-                t64[q] = t64_of(q, (double)kf[q]);
+                t64[q] = t64_of(q, (double)kf[q], inv);
                 t_next = fmin(t_next, t64[q]);
             }
-            const double len = sqrt(dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2]);
-            if (t_next > t_cur && (t_next - t_cur) * len >= 1e-9 * (double)vf && !mark_if_inside()) break;
+            // the interval's length against 1e-9 voxel: with the FP32 length of d
+            // unless that is within 1e-3 of the rule
+            const double span = (t_next - t_cur) * (double)len, rule = 1e-9 * (double)vf;
+            bool marks = t_next > t_cur && span >= 0.999 * rule;
+            if (marks && span <= 1.001 * rule)
+                marks = (t_next - t_cur) * sqrt(dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2]) >= rule;
+            if (marks && !mark_if_inside()) break;
             if (t_next >= t_end) break;
             float e = e_t;
 #pragma unroll
@@ -226,13 +255,15 @@ __global__ void __launch_bounds__(256) k_occ_rays(GridDev g, const DevCamera *ca
             cur_hi = (float)t_next + e;
         }
         flush();
+        mask = old_mask & ~old_bits;
+        if (mask) atomicOr(&free_bits[old_word], mask);
         // the end point's voxel: in FP32 unless a coordinate is within 1e-2 voxel
         // of a plane (its FP32 error is below 2^-20 of the distances involved)
         int ce[3];
         bool clear = true;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const float x = fmaf(te, (float)dv[a], -gf[a]) * g.inv_vox;
+            const float x = fmaf(te, d32[a], -gf[a]) * g.inv_vox;
             const float fl = floorf(x);
             if (!(x - fl >= 1e-2f && x - fl <= 0.99f && fabsf(x) < 8192.f)) clear = false;
             ce[a] = (int)fl;
@@ -325,9 +356,9 @@ void launch_occupancy_scan(const GridDev &g, const DevCamera *cams, int view, in
                            cudaStream_t s)
 {
     // one thread per pixel: the traversal lengths differ widely between rays
-    int blocks_r = (n_pix + 255) / 256;
+    int blocks_r = (n_pix + 127) / 128;
     if (blocks_r < 1) blocks_r = 1;
-    k_occ_rays<<<blocks_r, 256, 0, s>>>(g, cams, view, static_cast<const OccView *>(views), tab, depth, opacity, q.a_min,
+    k_occ_rays<<<blocks_r, 128, 0, s>>>(g, cams, view, static_cast<const OccView *>(views), tab, depth, opacity, q.a_min,
                                         hit, free_bits, hit_bits);
     const int64_t n_words = (int64_t)g.wpr * g.gy * g.gz;
     int64_t blocks_a = (n_words + 255) / 256;
