@@ -223,17 +223,18 @@ __global__ void __launch_bounds__(512) k_scatter(const uint32_t *cnt, const uint
     }
 }
 
-// tile t of the list: the last field whose first tile is <= t
+// tile t of the list: the last field whose first tile is <= t (plain loads: the
+// scan that writes both arrays may still run when this kernel is launched)
 __device__ __forceinline__ Tile tile_record(uint32_t t, const uint32_t *tile_off, const uint32_t *offsets, int n_fields,
                                             int tile)
 {
     int lo = 0, hi = n_fields - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(tile_off + mid) <= t) lo = mid; else hi = mid - 1;
+        if (tile_off[mid] <= t) lo = mid; else hi = mid - 1;
     }
-    const uint32_t k = t - __ldg(tile_off + lo);
-    const uint32_t o0 = __ldg(offsets + lo), h = __ldg(offsets + lo + 1) - o0;
+    const uint32_t k = t - tile_off[lo];
+    const uint32_t o0 = offsets[lo], h = offsets[lo + 1] - o0;
     Tile tl;
     tl.field = (uint32_t)lo;
     tl.start = o0 + k * (uint32_t)tile;

@@ -30,8 +30,10 @@ inline void raise_smem_limit(const void *kernel, int bytes, int (&cached)[kMaxDe
 // (a render round is five launches of a few microseconds each), so a kernel is
 // launched while its predecessor ends and starts with pdl_begin, which waits for
 // all of the predecessor's work and then lets its own successor be launched.
-// Nothing global is touched before it.  (After a launch of another kind, and
-// in a launch without the attribute, the order is the stream's.)
+// Nothing global is touched before it, and nothing that the predecessor writes
+// is read through read-only loads (__ldg, const __restrict__ parameters): those
+// ask for data that is constant from the kernel's launch on.  (After a launch of
+// another kind, and in a launch without the attribute, the order is the stream's.)
 __device__ __forceinline__ void pdl_begin()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
