@@ -61,24 +61,23 @@ __device__ __forceinline__ void st_words32(uint32_t tArow, int c, const uint32_t
     }
 }
 
-// Persistent kernel, one CTA per SM, kSlots tiles in flight.  Slot s is
-// warpgroup s (W = 128: warpgroups 2 s and 2 s + 1, each with half of every
-// row's columns): its threads encode and run the epilogues of their tile
-// (one row each), and one of them issues the tile's MMAs itself --
-// tcgen05.mma and tcgen05.commit occupy the issuing thread for tens to
-// hundreds of cycles each, so one issuer per slot lets the slots' chains
-// overlap.  Tiles come in field-uniform groups of kSlots (bucket padding);
+// Persistent kernel, one CTA per SM, kSlots tiles in flight.  Slot s is CG
+// warpgroups, each with its share of every row's columns: its threads encode
+// and run the epilogues of their tile (one row each), and one of them issues
+// the tile's MMAs itself -- tcgen05.mma and tcgen05.commit occupy the issuing
+// thread for tens to hundreds of cycles each, so one issuer per slot lets the
+// slots' chains overlap.  Tiles come in field-uniform groups of kSlots (bucket padding);
 // at a field change all slots meet at a CTA barrier, thread 0 reloads the
 // shared weight image, and each issuer waits for it before its next MMA.
-template <int W, int H, bool F8>
-__global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * TcShape<W, H, F8>::kSlotThreads, 1)
+template <int W, int H, bool F8, int CG>
+__global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * CG * 128, 1)
     k_mlp_tc(const void *wimg, int64_t img_bytes, int field_base, int cls, const float *affine, float sig_scale,
              int act, SampleSrc src, BucketBufs b, Counters *ctr, float4 *out, unsigned long long wait_ns,
              int withhold_image)
 {
     using S = TcShape<W, H, F8>;
     constexpr int kSlots = S::kSlots;
-    constexpr int CG = S::kColGroups, ST = S::kSlotThreads;
+    constexpr int ST = CG * 128;                     // threads of one slot
     constexpr int NC = W / CG;                       // columns of one warpgroup's share of a row
     constexpr int kLayers = S::kLayers;
     constexpr int kStageRec = kLayers >= 4 ? 1 : 0;  // the layer after which the next tile's records are gathered
@@ -147,10 +146,11 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * TcShape<W, H, F8>:
     Tile tl{0u, 0u, 0u, 0u};
     SampleIn nxt{0u, 0.f, 0.f, 0.f, 0.f, 0.f, 1.f};
     Pending pend{};
+    const SampleNeeds need{cg == 0, cg == CG - 1};
     uint32_t g = g0;
     if (g < g1) {
         tl = tiles[g * kSlots + slot];
-        nxt = fetch_sample(src, b, tl, row);
+        nxt = fetch_sample(src, b, tl, row, need);
     }
     for (; g < g1; ++g) {
         const uint32_t f = tl.field;           // identical for every slot (field-uniform groups)
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * TcShape<W, H, F8>:
         const SampleIn sm = nxt;
         if (g + 1 < g1) tl = tiles[(g + 1) * kSlots + slot];
         if (cur.count == 0) {
-            if (g + 1 < g1) nxt = fetch_sample(src, b, tl, row);
+            if (g + 1 < g1) nxt = fetch_sample(src, b, tl, row, need);
             continue;
         }
         const bool valid = (uint32_t)row < cur.count;
@@ -398,8 +398,8 @@ __global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * TcShape<W, H, F8>:
             }
             tc_fence_before();
             // each gather stage a layer or more after the load it depends on
-            if (l == kStageRec) stage_record(pend, src);
-            if (l == kLayers - 2) stage_ray(pend, src);
+            if (l == kStageRec) stage_record(pend, src, need);
+            if (l == kLayers - 2) stage_ray(pend, src, need);
         }
         if (!aborted) nxt = stage_finish(pend, src);
     }
@@ -516,18 +516,41 @@ __global__ void k_adam_tc(float *__restrict__ w, float *__restrict__ m, float *_
 template <int W, int H, bool F8>
 int tc_smem_bytes() { return 1024 + TcShape<W, H, F8>::kImageAlloc; }
 
-template <int W, int H, bool F8>
-void launch_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out, int n_sm,
-              cudaStream_t s)
+template <int W, int H, bool F8, int CG>
+void launch_cg(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out, int n_sm,
+               cudaStream_t s)
 {
     constexpr int kSlots = TcShape<W, H, F8>::kSlots;
     const int smem = tc_smem_bytes<W, H, F8>();
     static int smem_set[kMaxDevices] = {};
-    raise_smem_limit((const void *)k_mlp_tc<W, H, F8>, smem, smem_set);
+    raise_smem_limit((const void *)k_mlp_tc<W, H, F8, CG>, smem, smem_set);
     const void *img = F8 ? w.wimg8 : w.wimg;
     const int64_t ib = F8 ? w.img8_bytes : w.img_bytes;
-    launch_pdl(k_mlp_tc<W, H, F8>, n_sm, kSlots * TcShape<W, H, F8>::kSlotThreads, smem, s, img, ib, w.field_base, w.cls,
-               w.affine, w.sigma_scale, w.act, src, b, ctr, out, w.wait_ns ? w.wait_ns : kWaitNs, w.withhold_image);
+    launch_pdl(k_mlp_tc<W, H, F8, CG>, n_sm, kSlots * CG * 128, smem, s, img, ib, w.field_base, w.cls, w.affine,
+               w.sigma_scale, w.act, src, b, ctr, out, w.wait_ns ? w.wait_ns : kWaitNs, w.withhold_image);
+}
+
+// Warpgroups per slot.  TMEM admits only two slots at W = 128, whose epilogues
+// leave most issue slots empty with one warpgroup each; but two, at 128
+// registers a thread where one takes 152, hide less of a gather's latency.  FP8:
+// two (8.2 M samples of a render at H = 3 2009 -> 1952 us, 4 M scattered points
+// 1114 -> 1070).  BF16: two for rays, whose samples lie together in memory
+// (the same render 1940 -> 1852 us), one for direct points, which a caller may
+// have in any order (4 M scattered points of 128 fields at H = 4: 1135 us, 1245
+// with two; points in field order 1200 and 1117).
+template <int W, int H, bool F8>
+void launch_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out, int n_sm,
+              cudaStream_t s)
+{
+    if constexpr (W < 128) {
+        launch_cg<W, H, F8, 1>(w, src, b, ctr, out, n_sm, s);
+    } else if constexpr (F8) {
+        launch_cg<W, H, F8, 2>(w, src, b, ctr, out, n_sm, s);
+    } else {
+        // (the wait self-test runs the form with the longer way out)
+        if (src.mode == 0 || w.withhold_image) launch_cg<W, H, F8, 2>(w, src, b, ctr, out, n_sm, s);
+        else launch_cg<W, H, F8, 1>(w, src, b, ctr, out, n_sm, s);
+    }
 }
 
 #define ROAM_TC_CASES                                                                                   \

@@ -57,11 +57,6 @@ struct TcShape {
     // registers fit (6 x 128 threads: 80): 8.4 M samples at H = 2 take 446 us
     // with 6, 462 with 5, 552 with 4.
     static constexpr int kSlots = W == 32 ? 6 : (512 / kSlotCols >= 4 ? 4 : (512 / kSlotCols >= 2 ? 2 : 1));
-    // warpgroups per slot, each with its share of a row's columns: TMEM admits
-    // only two slots at W = 128, whose epilogues would leave most issue slots
-    // empty with one warpgroup each
-    static constexpr int kColGroups = kSlots >= 4 ? 1 : 2;
-    static constexpr int kSlotThreads = 128 * kColGroups;
 };
 
 // ---- PTX wrappers ----
@@ -408,7 +403,16 @@ struct Pending {
     float4 o, d;
 };
 
-__device__ __forceinline__ SampleIn fetch_sample(const SampleSrc &src, const BucketBufs &b, const Tile &tl, int row)
+// What a thread needs of its sample: with two warpgroups per slot the first
+// encodes the position and the second the direction, and each gathers its own
+// only (4 M scattered points at W = 128 / H = 4 in BF16, whose weight image
+// leaves L1 the least room: 1399 us with both gathering both, 1245 so).
+struct SampleNeeds {
+    bool pos, dir;
+};
+
+__device__ __forceinline__ SampleIn fetch_sample(const SampleSrc &src, const BucketBufs &b, const Tile &tl, int row,
+                                                 SampleNeeds need = {true, true})
 {
     SampleIn r{0u, 0.f, 0.f, 0.f, 0.f, 0.f, 1.f};
     if ((uint32_t)row >= tl.count) return r;
@@ -417,14 +421,17 @@ __device__ __forceinline__ SampleIn fetch_sample(const SampleSrc &src, const Buc
         const uint32_t col = r.idx >> 5;
         const uint32_t i = (col / (uint32_t)src.R) * 32u + (r.idx & 31u);
         const uint32_t ray = src.live ? src.live[i] : i;
-        const uint32_t j = src.recs[r.idx] & 0xffffu;
-        const float tt = ((float)j + 0.5f) * src.delta;
-        const float4 o = src.st.orig[ray], d = src.st.dir[ray];
-        r.px = fmaf(tt, d.x, o.x); r.py = fmaf(tt, d.y, o.y); r.pz = fmaf(tt, d.z, o.z);
+        const float4 d = src.st.dir[ray];
+        if (need.pos) {
+            const float tt = ((float)(src.recs[r.idx] & 0xffffu) + 0.5f) * src.delta;
+            const float4 o = src.st.orig[ray];
+            r.px = fmaf(tt, d.x, o.x); r.py = fmaf(tt, d.y, o.y); r.pz = fmaf(tt, d.z, o.z);
+        }
         r.dx = d.x; r.dy = d.y; r.dz = d.z;
     } else {
-        r.px = src.p[3 * (int64_t)r.idx]; r.py = src.p[3 * (int64_t)r.idx + 1]; r.pz = src.p[3 * (int64_t)r.idx + 2];
-        r.dx = src.d[3 * (int64_t)r.idx]; r.dy = src.d[3 * (int64_t)r.idx + 1]; r.dz = src.d[3 * (int64_t)r.idx + 2];
+        const int64_t k = 3 * (int64_t)r.idx;
+        if (need.pos) { r.px = src.p[k]; r.py = src.p[k + 1]; r.pz = src.p[k + 2]; }
+        if (need.dir) { r.dx = src.d[k]; r.dy = src.d[k + 1]; r.dz = src.d[k + 2]; }
     }
     return r;
 }
@@ -435,25 +442,25 @@ __device__ __forceinline__ void stage_index(Pending &q, const BucketBufs &b, con
     if (q.on) q.idx = b.sorted[tl.start + row];
 }
 
-__device__ __forceinline__ void stage_record(Pending &q, const SampleSrc &src)
+__device__ __forceinline__ void stage_record(Pending &q, const SampleSrc &src, SampleNeeds need = {true, true})
 {
     if (!q.on || src.mode != 0) return;
     const uint32_t col = q.idx >> 5;
     const uint32_t i = (col / (uint32_t)src.R) * 32u + (q.idx & 31u);
-    q.rec = src.recs[q.idx];
+    if (need.pos) q.rec = src.recs[q.idx];
     q.ray = src.live ? src.live[i] : i;
 }
 
-__device__ __forceinline__ void stage_ray(Pending &q, const SampleSrc &src)
+__device__ __forceinline__ void stage_ray(Pending &q, const SampleSrc &src, SampleNeeds need = {true, true})
 {
     if (!q.on) return;
     if (src.mode == 0) {
-        q.o = src.st.orig[q.ray];
+        if (need.pos) q.o = src.st.orig[q.ray];
         q.d = src.st.dir[q.ray];
     } else {
         const int64_t k = 3 * (int64_t)q.idx;
-        q.o = make_float4(src.p[k], src.p[k + 1], src.p[k + 2], 0.f);
-        q.d = make_float4(src.d[k], src.d[k + 1], src.d[k + 2], 0.f);
+        if (need.pos) q.o = make_float4(src.p[k], src.p[k + 1], src.p[k + 2], 0.f);
+        if (need.dir) q.d = make_float4(src.d[k], src.d[k + 1], src.d[k + 2], 0.f);
     }
 }
 
