@@ -9,6 +9,7 @@
 #include <vector>
 
 
+#include "dispatch.cuh"
 #include "internal.cuh"
 
 using namespace roam;
@@ -420,11 +421,10 @@ roam_status upload_cams(roam_ctx *c, const roam_camera *cams, int n_views, float
 }
 
 // tile records needed for `samples` samples in tiles of `tile`: each field's
-// run rounded up to its padding (at most 8, or the forced padding rounded up
-// to a kernel's tiles in flight)
+// run rounded up to its padding (of at most 6 tiles in flight)
 size_t tile_capacity(const roam_ctx *c, size_t samples, int tile = 128)
 {
-    return samples / (size_t)tile + (size_t)c->n_fields * (size_t)(c->tile_pad + 8) + 1;
+    return samples / (size_t)tile + (size_t)c->n_fields * (size_t)std::max(8, tile_run(c->tile_pad, 6)) + 1;
 }
 
 roam_status ensure_rays(roam_ctx *c, int64_t n_rays, int R)
@@ -505,8 +505,7 @@ ClassBounds classes_of(const roam_ctx *c, int precision)
     for (int k = 0; k < 4; ++k) {
         cb.group[k] = 1;
         if (precision == ROAM_F32 || k >= c->n_ws) continue;
-        const int g = tc_tile_group(c->ws[k].W, precision == ROAM_FP8);
-        cb.group[k] = std::max(1, (c->tile_pad + g - 1) / g) * g;
+        cb.group[k] = tile_run(c->tile_pad, tc_tile_group(c->ws[k].W, precision == ROAM_FP8));
     }
     return cb;
 }
@@ -1384,7 +1383,6 @@ roam_status roam_get_stats(roam_ctx *c, roam_stats *st)
 roam_status roam_set_tile_padding(roam_ctx *c, int tiles)
 {
     ROAM_TRY(set_dev(c));
-    // (each width class rounds it up to its own kernel's tiles in flight)
     if (tiles != 0 && (tiles < 4 || tiles > 64 || tiles % 4))
         return fail(ROAM_ERR_ARG, "tile padding must be 0 or a multiple of 4 in [4, 64]");
     c->tile_pad = tiles;
