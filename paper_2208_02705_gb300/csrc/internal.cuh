@@ -242,6 +242,7 @@ struct MlpWeights {
     int64_t img_bytes;
     const void *wimg8;         // FP8 E4M3 tensor-core images [F][img8_bytes]
     int64_t img8_bytes;
+    int slots;                 // tensor-core forward: tiles in flight per SM (tc_slots)
     int cls;                   // width class: the kernels take tiles [class_tiles[cls], class_tiles[cls + 1])
     int field_base;            // first internal field id of the class (row 0 of the per-class arrays)
     const float *affine;       // [F][6]
@@ -339,7 +340,6 @@ void set_error_message(const char *msg);
 bool tc_supported(int W, int H, bool f8);
 int64_t tc_image_bytes(int W, int H, bool f8);
 int tc_tile_samples();
-int tc_tile_group(int W, bool f8);
 // Adam fused with the BF16 image refresh (W <= 64); false: not available for this shape
 bool launch_adam_tc(float *w32, float *m, float *v, const float *g, int n_fields, int W, int H, int64_t P, void *wimg,
                     int64_t img_bytes, float lr, float b1, float b2, float eps, float bc1, float bc2, cudaStream_t s);

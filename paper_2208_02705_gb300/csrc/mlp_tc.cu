@@ -69,14 +69,13 @@ __device__ __forceinline__ void st_words32(uint32_t tArow, int c, const uint32_t
 // slots' chains overlap.  Tiles come in field-uniform groups of kSlots (bucket padding);
 // at a field change all slots meet at a CTA barrier, thread 0 reloads the
 // shared weight image, and each issuer waits for it before its next MMA.
-template <int W, int H, bool F8, int CG>
-__global__ void __launch_bounds__(TcShape<W, H, F8>::kSlots * CG * 128, 1)
+template <int W, int H, bool F8, int kSlots, int CG>
+__global__ void __launch_bounds__(kSlots * CG * 128, 1)
     k_mlp_tc(const void *wimg, int64_t img_bytes, int field_base, int cls, const float *affine, float sig_scale,
              int act, SampleSrc src, BucketBufs b, Counters *ctr, float4 *out, unsigned long long wait_ns,
              int withhold_image)
 {
     using S = TcShape<W, H, F8>;
-    constexpr int kSlots = S::kSlots;
     constexpr int ST = CG * 128;                     // threads of one slot
     constexpr int NC = W / CG;                       // columns of one warpgroup's share of a row
     constexpr int kLayers = S::kLayers;
@@ -516,21 +515,21 @@ __global__ void k_adam_tc(float *__restrict__ w, float *__restrict__ m, float *_
 template <int W, int H, bool F8>
 int tc_smem_bytes() { return 1024 + TcShape<W, H, F8>::kImageAlloc; }
 
-template <int W, int H, bool F8, int CG>
-void launch_cg(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out, int n_sm,
+template <int W, int H, bool F8, int kSlots, int CG>
+void launch_form(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out, int n_sm,
                cudaStream_t s)
 {
-    constexpr int kSlots = TcShape<W, H, F8>::kSlots;
     const int smem = tc_smem_bytes<W, H, F8>();
     static int smem_set[kMaxDevices] = {};
-    raise_smem_limit((const void *)k_mlp_tc<W, H, F8, CG>, smem, smem_set);
+    raise_smem_limit((const void *)k_mlp_tc<W, H, F8, kSlots, CG>, smem, smem_set);
     const void *img = F8 ? w.wimg8 : w.wimg;
     const int64_t ib = F8 ? w.img8_bytes : w.img_bytes;
-    launch_pdl(k_mlp_tc<W, H, F8, CG>, n_sm, kSlots * CG * 128, smem, s, img, ib, w.field_base, w.cls, w.affine,
+    launch_pdl(k_mlp_tc<W, H, F8, kSlots, CG>, n_sm, kSlots * CG * 128, smem, s, img, ib, w.field_base, w.cls, w.affine,
                w.sigma_scale, w.act, src, b, ctr, out, w.wait_ns ? w.wait_ns : kWaitNs, w.withhold_image);
 }
 
-// Warpgroups per slot.  TMEM admits only two slots at W = 128, whose epilogues
+// Tiles in flight (w.slots: as the tiles were padded) and warpgroups per slot.
+// TMEM admits only two slots at W = 128, whose epilogues
 // leave most issue slots empty with one warpgroup each; but two, at 128
 // registers a thread where one takes 152, hide less of a gather's latency.  FP8:
 // two (8.2 M samples of a render at H = 3 2009 -> 1952 us, 4 M scattered points
@@ -542,14 +541,17 @@ template <int W, int H, bool F8>
 void launch_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out, int n_sm,
               cudaStream_t s)
 {
-    if constexpr (W < 128) {
-        launch_cg<W, H, F8, 1>(w, src, b, ctr, out, n_sm, s);
+    if constexpr (W == 32) {
+        if (w.slots == 6) launch_form<W, H, F8, 6, 1>(w, src, b, ctr, out, n_sm, s);
+        else launch_form<W, H, F8, 4, 1>(w, src, b, ctr, out, n_sm, s);
+    } else if constexpr (W == 64) {
+        launch_form<W, H, F8, 4, 1>(w, src, b, ctr, out, n_sm, s);
     } else if constexpr (F8) {
-        launch_cg<W, H, F8, 2>(w, src, b, ctr, out, n_sm, s);
+        launch_form<W, H, F8, 2, 2>(w, src, b, ctr, out, n_sm, s);
     } else {
         // (the wait self-test runs the form with the longer way out)
-        if (src.mode == 0 || w.withhold_image) launch_cg<W, H, F8, 2>(w, src, b, ctr, out, n_sm, s);
-        else launch_cg<W, H, F8, 1>(w, src, b, ctr, out, n_sm, s);
+        if (src.mode == 0 || w.withhold_image) launch_form<W, H, F8, 2, 2>(w, src, b, ctr, out, n_sm, s);
+        else launch_form<W, H, F8, 2, 1>(w, src, b, ctr, out, n_sm, s);
     }
 }
 
@@ -579,13 +581,6 @@ int64_t tc_image_bytes(int W, int H, bool f8)
 }
 
 int tc_tile_samples() { return 128; }
-
-int tc_tile_group(int W, bool f8)
-{
-    if (W <= 32) return f8 ? TcShape<32, 1, true>::kSlots : TcShape<32, 1, false>::kSlots;
-    if (W <= 64) return f8 ? TcShape<64, 1, true>::kSlots : TcShape<64, 1, false>::kSlots;
-    return f8 ? TcShape<128, 1, true>::kSlots : TcShape<128, 1, false>::kSlots;
-}
 
 bool launch_adam_tc(float *w32, float *m, float *v, const float *g, int n_fields, int W, int H, int64_t P, void *wimg,
                     int64_t img_bytes, float lr, float b1, float b2, float eps, float bc1, float bc2, cudaStream_t s)

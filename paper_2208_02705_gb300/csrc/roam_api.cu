@@ -494,28 +494,36 @@ bool adjoint_on_tc(const roam_ctx *c, int precision)
 }
 
 int tile_of(int precision) { return precision != ROAM_F32 ? tc_tile_samples() : 128; }
+// The tensor-core forward's tiles in flight for class k of a launch over about
+// `samples` samples (spread over the fields alike).
+int slots_of(const roam_ctx *c, int k, int64_t samples)
+{
+    return tc_slots(c->ws[k].W, samples * c->ws[k].n / std::max(1, c->n_fields), c->ws[k].n, c->n_sm);
+}
+
 // The classes with the tile padding of their MLP kernels: on the tensor cores
-// every field's tile run is a multiple of its own kernel's tiles in flight
-// (6 / 4 / 2 at W = 32 / 64 / 128), so that no group of tiles is empty
-// throughout and a class's groups, counted from its first tile, never mix
-// fields.  FP32 (SIMT, one tile at a time): no padding.
-ClassBounds classes_of(const roam_ctx *c, int precision)
+// every field's tile run is a multiple of its own kernel's tiles in flight, so
+// that no group of tiles is empty throughout and a class's groups, counted from
+// its first tile, never mix fields.  FP32 (SIMT, one tile at a time): no padding.
+ClassBounds classes_of(const roam_ctx *c, int precision, int64_t samples)
 {
     ClassBounds cb = c->cb;
     for (int k = 0; k < 4; ++k) {
         cb.group[k] = 1;
         if (precision == ROAM_F32 || k >= c->n_ws) continue;
-        cb.group[k] = tile_run(c->tile_pad, tc_tile_group(c->ws[k].W, precision == ROAM_FP8));
+        cb.group[k] = tile_run(c->tile_pad, slots_of(c, k, samples));
     }
     return cb;
 }
 
-roam_status run_mlp(roam_ctx *c, int precision, const SampleSrc &src, const BucketBufs &b, float4 *out,
-                    Counters *ctr, cudaStream_t s)
+// (samples: as in the classes_of of the bucketing before it)
+roam_status run_mlp(roam_ctx *c, int precision, int64_t samples, const SampleSrc &src, const BucketBufs &b,
+                    float4 *out, Counters *ctr, cudaStream_t s)
 {
     // one launch per width class over its own tile range
     for (int k = 0; k < c->n_ws; ++k) {
-        const MlpWeights w = weights_of(c, k);
+        MlpWeights w = weights_of(c, k);
+        w.slots = slots_of(c, k, samples);
         if (precision != ROAM_F32) {
             launch_mlp_tc(w, precision == ROAM_FP8, src, b, ctr, out, c->n_sm, s);
             ROAM_TRY(launched("mlp_tc"));
@@ -560,6 +568,7 @@ roam_status run_rounds(roam_ctx *c, const uint32_t *rays, int64_t n_rays, const 
         mp.init = r == 0;
         mp.live = r == 0 ? nullptr : lives[r & 1];
         mp.live_count = r == 0 ? nullptr : &c->ctr->live_count[r & 1];
+        const int64_t samples = round_samples(n_rays, Rr, r == 0);
         {
             ProfScope ps(c, P_MARCH, s);
             launch_march(c->g, mp, march_grid(mp.n_rays), s);
@@ -568,7 +577,7 @@ roam_status run_rounds(roam_ctx *c, const uint32_t *rays, int64_t n_rays, const 
         {
             ProfScope ps(c, P_BUCKET, s);
             launch_bucket_ready(mp.cnt, mp.recs, mp.live_count, mp.n_rays, Rr, 1, c->n_fields, tile_of(o->precision), b,
-                                c->ctr, grid, s, classes_of(c, o->precision));
+                                c->ctr, grid, s, classes_of(c, o->precision, samples));
         }
         ROAM_TRY(launched("bucket"));
         SampleSrc src{};
@@ -582,7 +591,7 @@ roam_status run_rounds(roam_ctx *c, const uint32_t *rays, int64_t n_rays, const 
         src.accurate = mp.accurate;
         {
             ProfScope ps(c, o->precision == ROAM_BF16 ? P_MLP_BF16 : (o->precision == ROAM_FP8 ? P_MLP_FP8 : P_MLP_F32), s);
-            ROAM_TRY(run_mlp(c, o->precision, src, b, c->sr.p, c->ctr, s));
+            ROAM_TRY(run_mlp(c, o->precision, samples, src, b, c->sr.p, c->ctr, s));
         }
         {
             ProfScope ps(c, P_COMPOSITE, s);
@@ -1410,7 +1419,7 @@ roam_status roam_selftest_wait_timeout(roam_ctx *c, uint64_t limit_ns, int32_t *
     const BucketBufs b = bucket_of(c);
     ROAM_CUDA(cudaMemsetAsync(c->aux, 0, sizeof(Counters), s));
     launch_bucket(nullptr, nullptr, nullptr, (uint32_t)n, 1, 1, keys, c->n_fields, tile_of(ROAM_BF16), b, c->aux,
-                  grid_blocks(c, 2), s, classes_of(c, ROAM_BF16));
+                  grid_blocks(c, 2), s, classes_of(c, ROAM_BF16, n));
     ROAM_TRY(launched("bucket"));
     SampleSrc src{};
     src.mode = 1;
@@ -1419,6 +1428,7 @@ roam_status roam_selftest_wait_timeout(roam_ctx *c, uint64_t limit_ns, int32_t *
     MlpWeights w = weights_of(c, 0);
     w.wait_ns = limit_ns;
     w.withhold_image = 1;
+    w.slots = slots_of(c, 0, n);
     launch_mlp_tc(w, false, src, b, c->aux, reinterpret_cast<float4 *>(out), c->n_sm, s);
     ROAM_TRY(launched("mlp_tc"));
     ROAM_CUDA(cudaStreamSynchronize(s));
@@ -1558,14 +1568,14 @@ roam_status roam_mlp_eval(roam_ctx *c, const float *p, const float *d, const uin
         keys = c->keys_tmp.p;
     }
     launch_bucket(nullptr, nullptr, nullptr, (uint32_t)n, 1, 1, keys, c->n_fields, tile_of(precision), b, c->aux,
-                  grid_blocks(c, 2), s, classes_of(c, precision));
+                  grid_blocks(c, 2), s, classes_of(c, precision, n));
     ROAM_TRY(launched("bucket"));
     SampleSrc src{};
     src.mode = 1;
     src.p = p;
     src.d = d;
     c->last = s;
-    return run_mlp(c, precision, src, b, reinterpret_cast<float4 *>(out), c->aux, s);
+    return run_mlp(c, precision, n, src, b, reinterpret_cast<float4 *>(out), c->aux, s);
 }
 
 roam_status roam_composite(roam_ctx *c, int64_t n_rays, int n_max, const uint32_t *count, const float *sigma_rgb,

@@ -52,11 +52,6 @@ struct TcShape {
     static constexpr int kDCols = N_HEAD;
     static constexpr int kACols = K_COL * kEB / 4;
     static constexpr int kSlotCols = kDCols + kACols;
-    // Tiles in flight: what TMEM admits.  At W = 32 a layer is mostly the slot's
-    // barrier, commit round trip and waits, so more slots pay as long as their
-    // registers fit (6 x 128 threads: 80): 8.4 M samples at H = 2 take 446 us
-    // with 6, 462 with 5, 552 with 4.
-    static constexpr int kSlots = W == 32 ? 6 : (512 / kSlotCols >= 4 ? 4 : (512 / kSlotCols >= 2 ? 2 : 1));
 };
 
 // ---- PTX wrappers ----
