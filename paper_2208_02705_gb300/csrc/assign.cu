@@ -20,20 +20,19 @@
 // (up to four per thread), histograms are pushed into every block's copy
 // through distributed shared memory, so a network costs four cluster barriers
 // and a few L2 latencies, and touches about as many voxels as it takes (instead
-// of every unassigned voxel five times in five launches).
+// of every unassigned voxel once per launch of the general form).
 //
 // The general form, for larger networks: per network
-//   k_hist_select  per digit of the 47-bit key (squared distance << 27 |
-//                  rank), a histogram of the candidates matching the digits
+//   k_hist_select  per digit of the key (squared distance << 27 | rank), a histogram of the candidates matching the digits
 //                  fixed so far (shared-memory bins, then global atomics);
 //                  the block that finishes last picks the bin holding the
 //                  wanted rank, growing the key prefix by one digit (4
-//                  digits of 12 bits)
+//                  digits of 12 bits; 5 where squared distances reach 2^21)
 //   k_take_anchor  every unassigned voxel whose key is <= the selected key
 //                  joins the network; the block that finishes last finds the
 //                  next network's anchor (the first unassigned voxel from a
 //                  cursor; k_anchor for the first network)
-// Five launches per network, with no waiting between blocks: the serial
+// Five or six launches per network, with no waiting between blocks: the serial
 // parts run in whichever block finishes last (a counter of finished blocks).
 // Keys are unique (the rank is part of them), so exactly s voxels are taken.
 // All state stays on the device: no host synchronisation per network.
@@ -135,19 +134,18 @@ __device__ __forceinline__ unsigned long long key_of(const AssignState &st, uint
     return (d2 << kRankBits) | rank;
 }
 
-// Histogram of digit `pass` (0 = most significant) of the keys matching the
-// prefix (shared-memory bins, then global atomics); then, in the block that
-// finishes last, the select: the bin holding rank_left extends the prefix by
-// one digit (512 threads, 8 bins each), and the histogram is cleared.
+// Histogram of the keys' digit at `shift` (`first`: the most significant) over
+// the keys matching the prefix (shared-memory bins, then global atomics); then,
+// in the block that finishes last, the select: the bin holding rank_left extends
+// the prefix by one digit (512 threads, 8 bins each), and the histogram is cleared.
 __global__ void __launch_bounds__(512) k_hist_select(const uint16_t *field, uint32_t S, const uint32_t *vox, int gx,
-                                                     int gy, AssignState *st, int pass, uint32_t *hist)
+                                                     int gy, AssignState *st, int shift, bool first, uint32_t *hist)
 {
     __shared__ uint32_t sh[kBins];
     for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0u;
     __syncthreads();
     {
         const AssignState sv = *st;
-        const int shift = (3 - pass) * kDigitBits;
         // eight candidates per thread per round, their loads issued together
         // (one dependent load after another per voxel would leave the SMs
         // waiting on L2 latency)
@@ -171,7 +169,7 @@ __global__ void __launch_bounds__(512) k_hist_select(const uint16_t *field, uint
                 const uint32_t i = i0 + (uint32_t)u * stride;
                 if (fv[u] != kFree || i >= S) continue;
                 const unsigned long long k = key_of(sv, vv[u], i, gx, gy);
-                if (pass > 0 && (k >> (shift + kDigitBits)) != sv.prefix) continue;
+                if (!first && (k >> (shift + kDigitBits)) != sv.prefix) continue;
                 atomicAdd(&sh[(k >> shift) & (kBins - 1)], 1u);
             }
         }
@@ -695,14 +693,17 @@ void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, 
         k_brick_lists<<<n_sm * 8, 256, 0, s>>>(cells, gx, gy, gz, L);
         k_assign_bricks<<<kCluster, kAT, 0, s>>>(field, S, vox, gx, gy, st, L, n, per);
     } else if (n > 1) {
-        // per network: 4 digit passes (histogram, then the select in the block
-        // that finishes last) and the take (then the next anchor, likewise)
+        // per network: a pass per digit (histogram, then the select in the block
+        // that finishes last) and the take (then the next anchor, likewise);
+        // 4 digits hold squared distances below 2^21, larger grids take 5
+        const uint64_t far = (uint64_t)gx * gx + (uint64_t)gy * gy + (uint64_t)gz * gz;
+        const int n_digits = far >> (4 * kDigitBits - kRankBits) ? 5 : 4;
         k_anchor<<<1, 1024, 0, s>>>(field, S, vox, gx, gy, st, per - 1u);
         for (int k = 0; k + 1 < n; ++k) {
             // one block per SM: fewer blocks flushing their shared histograms
             // (the first digits fall in a few bins, whose global atomics collide)
-            for (int pass = 0; pass < 4; ++pass)
-                k_hist_select<<<n_sm, 512, 0, s>>>(field, S, vox, gx, gy, st, pass, hist);
+            for (int d = n_digits - 1; d >= 0; --d)
+                k_hist_select<<<n_sm, 512, 0, s>>>(field, S, vox, gx, gy, st, d * kDigitBits, d == n_digits - 1, hist);
             k_take_anchor<<<grid, 1024, 0, s>>>(field, S, vox, gx, gy, st, (uint16_t)k, per - 1u);
         }
     }
