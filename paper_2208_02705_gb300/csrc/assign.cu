@@ -9,22 +9,25 @@
 // the earlier ones took), so what counts is the latency of one network.  Two
 // forms:
 //
-// k_assign_bricks (networks of up to kBrickMaxPer voxels): one cluster of 8
-// blocks builds every network in one launch.  The unassigned voxels are kept
-// in lists by 8^3 brick (each block owns every eighth brick).  Per network: a
+// k_assign_bricks (small networks of voxels that lie together; the line is
+// assign_from_bricks): one cluster of 8 blocks builds every network in one
+// launch.  The unassigned voxels are kept in lists by 8^3 brick (each block owns
+// every eighth brick).  Per network: a
 // histogram of the bricks' largest distance to the anchor, weighted by their
 // voxels, bounds the distance of the last voxel wanted; only bricks that reach
 // below that bound are candidates; a histogram of their voxels' squared
 // distances narrows the last voxel's key to one bin, and that bin's keys are
 // ranked directly.  The candidates' keys stay in registers between these steps
-// (up to four per thread), histograms are pushed into every block's copy
+// (up to four per thread; else they are formed again, a thread per brick of a
+// few voxels, a warp per brick of many), histograms are pushed into every block's copy
 // through distributed shared memory, so a network costs four cluster barriers
 // and a few L2 latencies, and touches about as many voxels as it takes (instead
 // of every unassigned voxel once per launch of the general form).
 //
-// The general form, for larger networks: per network
-//   k_hist_select  per digit of the key (squared distance << 27 | rank), a histogram of the candidates matching the digits
-//                  fixed so far (shared-memory bins, then global atomics);
+// The general form, for larger networks and scattered voxels: per network
+//   k_hist_select  per digit of the key (squared distance << 27 | rank), a
+//                  histogram of the candidates matching the digits fixed so
+//                  far (shared-memory bins, then global atomics);
 //                  the block that finishes last picks the bin holding the
 //                  wanted rank, growing the key prefix by one digit (4
 //                  digits of 12 bits; 5 where squared distances reach 2^21)
@@ -38,6 +41,7 @@
 // All state stays on the device: no host synchronisation per network.
 #include <cooperative_groups.h>
 
+#include "dispatch.cuh"
 #include "internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -291,6 +295,7 @@ struct BrickLists {
     uint32_t *coord;       // [NB] bx | by << 8 | bz << 16 (grids are at most 2048^3: 256 bricks per axis)
     uint32_t *count;       // [NB] unassigned voxels
     uint32_t *start;       // [NB] first entry
+    uint32_t *spill;       // [NB + 8] candidate bricks past a block's table (ceil(NB / 8) words per block)
     uint32_t *rank;        // [S] ranks, brick after brick
     uint16_t *loc;         // [S] voxel within its brick: x | y << 3 | z << 6
 };
@@ -387,6 +392,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
     __shared__ uint32_t cand[kCandMax], cand_at[kCandMax], cand_kept[kCandMax];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster.block_rank(), n_bricks = L.n[0];
+    uint32_t *const spill = L.spill + rank * ((n_bricks + kCluster - 1) / kCluster);
 
     hist[tid] = sum[0][tid] = sum[1][tid] = 0u;
     if (tid == 0) {
@@ -492,13 +498,15 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
                 cand[q] = b;
                 cand_at[q] = (uint32_t)at;
                 cand_kept[q] = 0u;
+            } else {
+                spill[q] = b;
             }
         }
         __syncthreads();
         const uint32_t nc = (uint32_t)(cand_s >> 32), nv = (uint32_t)cand_s;
-        const bool table = nc <= (uint32_t)kCandMax;
+        auto cand_of = [&](uint32_t q) { return q < (uint32_t)kCandMax ? cand[q] : spill[q]; };
         // a few voxels per thread: their keys stay in registers
-        const bool few = table && nv <= kVox * (uint32_t)kAT;
+        const bool few = nc <= (uint32_t)kCandMax && nv <= kVox * (uint32_t)kAT;
         unsigned long long vk[kVox];
         uint32_t vq[kVox];
         uint16_t vl[kVox];
@@ -522,41 +530,45 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
                 vl[u] = (uint16_t)l;
             }
         }
-        // else a warp goes over its block's candidates (past the table: over all
-        // of its block's bricks)
-        const uint32_t n_own = n_bricks > rank ? (n_bricks - rank + kCluster - 1) / kCluster : 0u;
-        const uint32_t n_it = table ? nc : n_own;
-        // every candidate voxel of this warp's bricks: f(brick, voxels, first entry, key of an entry)
-        auto visit = [&](auto f) {
-            for (uint32_t q = (uint32_t)warp; q < n_it; q += kAT / 32) {
-                const uint32_t b = table ? cand[q] : rank + q * kCluster;
-                const uint32_t c = L.coord[b], cnt = L.count[b], s0 = L.start[b];
-                if (!table) {
-                    uint32_t lo, hi;
-                    reach(c, lo, hi);
-                    if (lo >= bound) continue;
-                }
-                const int x0 = (int)(c & 255u) * 8 - ax, y0 = (int)((c >> 8) & 255u) * 8 - ay,
-                          z0 = (int)((c >> 16) & 255u) * 8 - az;
-                f(b, cnt, s0, [&](uint32_t e) -> unsigned long long {
-                    const uint32_t l = L.loc[e];
-                    const int dx = x0 + (int)(l & 7u), dy = y0 + (int)((l >> 3) & 7u), dz = z0 + (int)(l >> 6);
-                    return (unsigned long long)(uint32_t)(dx * dx + dy * dy + dz * dz) << kRankBits | L.rank[e];
-                });
-            }
+        // a brick's voxels as keys
+        struct Brick {
+            uint32_t n, first;
+            int x, y, z;
         };
+        auto open = [&](uint32_t b) {
+            const uint32_t c = L.coord[b];
+            return Brick{L.count[b], L.start[b], (int)(c & 255u) * 8 - ax, (int)((c >> 8) & 255u) * 8 - ay,
+                         (int)((c >> 16) & 255u) * 8 - az};
+        };
+        auto key = [&](const Brick &o, uint32_t e) -> unsigned long long {
+            const uint32_t l = L.loc[e];
+            const int dx = o.x + (int)(l & 7u), dy = o.y + (int)((l >> 3) & 7u), dz = o.z + (int)(l >> 6);
+            return (unsigned long long)(uint32_t)(dx * dx + dy * dy + dz * dz) << kRankBits | L.rank[e];
+        };
+        // else a thread goes over each of its block's candidates where these hold
+        // a few voxels each, a warp where they hold many
+        const bool sparse = nv < 6u * nc;
         auto each_key = [&](auto f) {
             if (few) {
 #pragma unroll
                 for (int u = 0; u < kVox; ++u)
                     if (vk[u] < bound_key) f(vk[u]);
-            } else {
-                visit([&](uint32_t, uint32_t cnt, uint32_t s0, auto key) {
-                    for (uint32_t e = (uint32_t)lane; e < cnt; e += 32) {
-                        const unsigned long long k = key(s0 + e);
+            } else if (sparse) {
+                for (uint32_t q = (uint32_t)tid; q < nc; q += kAT) {
+                    const Brick o = open(cand_of(q));
+                    for (uint32_t e = o.first; e < o.first + o.n; ++e) {
+                        const unsigned long long k = key(o, e);
                         if (k < bound_key) f(k);
                     }
-                });
+                }
+            } else {
+                for (uint32_t q = (uint32_t)warp; q < nc; q += kAT / 32) {
+                    const Brick o = open(cand_of(q));
+                    for (uint32_t e = (uint32_t)lane; e < o.n; e += 32) {
+                        const unsigned long long k = key(o, o.first + e);
+                        if (k < bound_key) f(k);
+                    }
+                }
             }
         };
         each_key([&](unsigned long long k) { atomicAdd(&hist[(uint32_t)(k >> (kRankBits + sh))], 1u); });
@@ -623,20 +635,22 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
             }
             __syncthreads();
             for (uint32_t q = (uint32_t)tid; q < nc; q += kAT) L.count[cand[q]] = cand_kept[q];
-        } else {
-            visit([&](uint32_t b, uint32_t cnt, uint32_t s0, auto key) {
+        } else if (!sparse) {
+            for (uint32_t q = (uint32_t)warp; q < nc; q += kAT / 32) {
+                const uint32_t b = cand_of(q);
+                const Brick o = open(b);
                 uint32_t kept = 0;
-                for (uint32_t e0 = 0; e0 < cnt; e0 += 32) {
-                    const uint32_t e = s0 + e0 + (uint32_t)lane;
-                    const bool in = e0 + (uint32_t)lane < cnt;
+                for (uint32_t e0 = 0; e0 < o.n; e0 += 32) {
+                    const uint32_t e = o.first + e0 + (uint32_t)lane;
+                    const bool in = e0 + (uint32_t)lane < o.n;
                     const uint32_t r = in ? L.rank[e] : 0u;
                     const uint16_t l = in ? L.loc[e] : (uint16_t)0;
-                    const bool take = in && key(in ? e : s0) <= thr;
+                    const bool take = in && key(o, in ? e : o.first) <= thr;
                     const unsigned km = __ballot_sync(0xffffffffu, in && !take);
                     if (take) __stcg(&field[r], (uint16_t)net);
                     __syncwarp();
                     if (in && !take) {
-                        const uint32_t at = s0 + kept + (uint32_t)__popc(km & ((1u << lane) - 1u));
+                        const uint32_t at = o.first + kept + (uint32_t)__popc(km & ((1u << lane) - 1u));
                         L.rank[at] = r;
                         L.loc[at] = l;
                     }
@@ -644,7 +658,25 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
                     kept += (uint32_t)__popc(km);
                 }
                 if (lane == 0) L.count[b] = kept;
-            });
+            }
+        } else {
+            for (uint32_t q = (uint32_t)tid; q < nc; q += kAT) {
+                const uint32_t b = cand_of(q);
+                const Brick o = open(b);
+                uint32_t kept = 0;
+                for (uint32_t e = o.first; e < o.first + o.n; ++e) {
+                    const uint32_t r = L.rank[e];
+                    const uint16_t l = L.loc[e];
+                    if (key(o, e) <= thr) {
+                        __stcg(&field[r], (uint16_t)net);
+                    } else {
+                        L.rank[o.first + kept] = r;
+                        L.loc[o.first + kept] = l;
+                        ++kept;
+                    }
+                }
+                L.count[b] = kept;
+            }
         }
         __syncthreads();
         if (tid == 0) cand_s = 0ull;
@@ -656,20 +688,14 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
 
 }  // namespace
 
-// Networks up to this many voxels are built from the brick lists.  Measured per
-// network (GB300): 11 us against 52 us for the general form at 2,000 voxels,
-// 56 us at 33,000, where the general form takes 155; from 65,000 on, 8 blocks
-// against the whole chip, the two meet (89 us general at 67,000).
-constexpr uint32_t kBrickMaxPer = 65536u;
-
 // state and histogram, then (for the brick form) the lists
 size_t assign_scratch_bytes(uint32_t S, int64_t n_bricks)
 {
-    const size_t nb = (size_t)(n_bricks < (int64_t)S ? n_bricks : (int64_t)S);
-    return sizeof(AssignState) + kBins * sizeof(uint32_t) + 16 + nb * 12 + (size_t)S * 6;
+    const size_t nb = (size_t)n_bricks;
+    return sizeof(AssignState) + kBins * sizeof(uint32_t) + 16 + nb * 16 + 4 * kCluster + (size_t)S * 6;
 }
 
-void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, uint32_t S,
+void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, uint32_t S, int64_t n_bricks,
                    int n, uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm, cudaStream_t s)
 {
     AssignState *st = reinterpret_cast<AssignState *>(scratch);
@@ -680,15 +706,15 @@ void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, 
     k_occupied_list<<<n_sm * 8, 256, 0, s>>>(cells, n_words, vox);
     const uint32_t per = S / (uint32_t)n;
     const int grid = n_sm * 4;
-    if (n > 1 && per <= kBrickMaxPer) {
-        const int64_t n_bricks = (int64_t)(gx >> 3) * (gy >> 3) * (gz >> 3);
-        const size_t nb = (size_t)(n_bricks < (int64_t)S ? n_bricks : (int64_t)S);
+    if (n > 1 && assign_from_bricks(S, n_bricks, per)) {
+        const size_t nb = (size_t)n_bricks;
         BrickLists L;
         L.n = hist + kBins;
         L.coord = L.n + 4;
         L.count = L.coord + nb;
         L.start = L.count + nb;
-        L.rank = L.start + nb;
+        L.spill = L.start + nb;
+        L.rank = L.spill + nb + kCluster;
         L.loc = reinterpret_cast<uint16_t *>(L.rank + S);
         k_brick_lists<<<n_sm * 8, 256, 0, s>>>(cells, gx, gy, gz, L);
         k_assign_bricks<<<kCluster, kAT, 0, s>>>(field, S, vox, gx, gy, st, L, n, per);

@@ -35,6 +35,25 @@ constexpr int tc_slots(int W, int64_t samples, int n_fields, int n_sm)
     return samples >= 28 * 128 * (int64_t)n_fields && samples >= 16 * 128 * (int64_t)n_sm ? 6 : 4;
 }
 
+// Whether a map of S occupied voxels in `bricks` non-empty 8^3 bricks, split into
+// networks of `per` voxels, is assigned from brick lists (one cluster of 8 blocks
+// builds every network) or by the general form (whole-chip passes over all
+// unassigned voxels, five launches per network).  Microseconds per network of
+// either, fitted to both forms on the same maps (GB300; the first term of the
+// one is its cluster barriers, of the other its launches).  Measured, lists and
+// general:
+//   1.5 M voxels in 18,944 bricks:    33,000 per network   49 /  74, 139,000 133 / 109
+//   6.2 M in 86,528:                  15,500               34 / 115, 269,000 274 / 212
+//   262 k in 512:                      8,200               29 /  52, 131,000  77 /  62
+//   268 k in 168,116 (1.6 per brick):  2,000               35 /  50,  16,700 118 /  58
+//   2.0 M in 1,289,647:                5,000              150 /  84
+constexpr bool assign_from_bricks(int64_t S, int64_t bricks, int64_t per)
+{
+    const double lists = 10.0 + 1.2e-4 * (double)bricks + (double)per * (0.8e-3 + 8e-3 * (double)bricks / (double)S);
+    const double general = 44.0 + 1.15e-5 * (double)S + 3.3e-4 * (double)per;
+    return lists <= general;
+}
+
 // Samples that a round of a render marches, about: a ray of a mapped scene
 // keeps up to 16 in its first round, and an eighth of the rays go on.
 constexpr int64_t round_samples(int64_t n_rays, int round_size, bool first)

@@ -256,7 +256,9 @@ struct MlpWeights {
 // ---- kernels launched from the API layer -------------------------------
 
 void launch_grid_cells(const uint32_t *bits, uint2 *cells, uint32_t *block_sums, int64_t n_words, cudaStream_t s);
-void launch_brick_dist(GridDev g, uint8_t *occ, uint16_t *t0, uint16_t *t1, uint8_t *dist, cudaStream_t s);
+// (*n_occ, zero before, receives the number of occupied bricks)
+void launch_brick_dist(GridDev g, uint8_t *occ, uint16_t *t0, uint16_t *t1, uint8_t *dist, uint32_t *n_occ,
+                       cudaStream_t s);
 void launch_march(const GridDev &g, const MarchParams &p, int grid, cudaStream_t s);
 struct TeacherAffine {
     float v[6];      // global position -> [-1, 1]^3: scale xyz, offset xyz
@@ -273,7 +275,8 @@ void launch_teacher_simt(const float *wt, TeacherAffine aff, int64_t n, const fl
 void launch_distill_loss(int64_t n, const float4 *student, const float4 *teacher, float I, float4 *dl, float *loss,
                          cudaStream_t s);
 size_t assign_scratch_bytes(uint32_t S, int64_t n_bricks);
-void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, uint32_t S,
+// n_bricks: 8^3 bricks with an occupied voxel
+void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, uint32_t S, int64_t n_bricks,
                    int n, uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm, cudaStream_t s);
 uint32_t assign_status(const void *scratch);
 size_t occupancy_view_bytes(int n_views);

@@ -80,10 +80,11 @@ __global__ void k_prefix_add(uint2 *cells, const uint32_t *block_sums, int64_t n
     if (i < n_words) cells[i].y += block_sums[i / 4096];
 }
 
-// one thread per 8^3 brick: 1 if any of its 512 voxels is occupied
-__global__ void k_brick_occ(GridDev g, uint8_t *occ)
+// one thread per 8^3 brick: 1 if any of its 512 voxels is occupied; *n_occ += those
+__global__ void k_brick_occ(GridDev g, uint8_t *occ, uint32_t *n_occ)
 {
     const int64_t n = (int64_t)g.bx * g.by * g.bz;
+    uint32_t mine = 0;
     for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
         const int bx = (int)(b % g.bx), by = (int)((b / g.bx) % g.by), bz = (int)(b / ((int64_t)g.bx * g.by));
         const int x0 = bx << kBrickShift;
@@ -94,7 +95,10 @@ __global__ void k_brick_occ(GridDev g, uint8_t *occ)
                 any |= (w >> (x0 & 31)) & 0xffu;
             }
         occ[b] = any ? 1 : 0;
+        mine += any ? 1u : 0u;
     }
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if ((threadIdx.x & 31u) == 0 && mine) atomicAdd(n_occ, mine);
 }
 
 // Chebyshev (L-infinity) distance, in bricks, from every brick to the nearest
@@ -434,11 +438,12 @@ void launch_grid_cells(const uint32_t *bits, uint2 *cells, uint32_t *block_sums,
     k_prefix_add<<<(unsigned)((n_words + 255) / 256), 256, 0, s>>>(cells, block_sums, n_words);
 }
 
-void launch_brick_dist(GridDev g, uint8_t *occ, uint16_t *t0, uint16_t *t1, uint8_t *dist, cudaStream_t s)
+void launch_brick_dist(GridDev g, uint8_t *occ, uint16_t *t0, uint16_t *t1, uint8_t *dist, uint32_t *n_occ,
+                       cudaStream_t s)
 {
     const int64_t n = (int64_t)g.bx * g.by * g.bz;
     const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-    k_brick_occ<<<blocks, 256, 0, s>>>(g, occ);
+    k_brick_occ<<<blocks, 256, 0, s>>>(g, occ, n_occ);
     k_brick_dist<<<blocks, 256, 0, s>>>(g, 0, occ, nullptr, t0);
     k_brick_dist<<<blocks, 256, 0, s>>>(g, 1, occ, t0, t1);
     k_brick_dist<<<blocks, 256, 0, s>>>(g, 2, occ, t1, t0);

@@ -113,7 +113,7 @@ struct roam_ctx {
     bool has_grid = false;
     roam_grid_desc gd{};
     GridDev g{};
-    int64_t n_words = 0, n_occ = 0;
+    int64_t n_words = 0, n_occ = 0, n_bricks = 0;      // bit words; occupied voxels; bricks that hold one
     DBuf<uint32_t> bits, block_sums;
     DBuf<uint2> cells;                      // the bit words beside their rank prefixes
     DBuf<uint8_t> brick_occ, brick_dist;
@@ -909,11 +909,15 @@ roam_status roam_load_grid(roam_ctx *c, const roam_grid_desc *desc, const uint32
     g.n_fields = 0;
     launch_grid_cells(c->bits.p, c->cells.p, c->block_sums.p, n_words, 0);
     ROAM_TRY(launched("grid prefix"));
-    launch_brick_dist(g, c->brick_occ.p, c->brick_t0.p, c->brick_t1.p, c->brick_dist.p, 0);
+    ROAM_CUDA(cudaMemset(c->d_flag, 0, 4));
+    launch_brick_dist(g, c->brick_occ.p, c->brick_t0.p, c->brick_t1.p, c->brick_dist.p, c->d_flag, 0);
     ROAM_TRY(launched("brick distance map"));
+    uint32_t occ_bricks = 0;
+    ROAM_CUDA(cudaMemcpy(&occ_bricks, c->d_flag, 4, cudaMemcpyDeviceToHost));
     uint2 last{};
     ROAM_CUDA(cudaMemcpy(&last, c->cells.p + n_words - 1, sizeof(last), cudaMemcpyDeviceToHost));
     c->n_words = n_words;
+    c->n_bricks = (int64_t)occ_bricks;
     c->n_occ = (int64_t)last.y + __builtin_popcount(last.x);
     c->gd = *desc;
     c->has_grid = true;
@@ -1254,9 +1258,9 @@ roam_status roam_assign_fields(roam_ctx *c, int n_fields, uint16_t *labels, int3
     if (S >= (int64_t)1 << 27) return fail(ROAM_ERR_ARG, "at most 2^27 - 1 occupied voxels");
     cudaStream_t s = (cudaStream_t)stream;
     ROAM_TRY(ensure(c->assign_vox, (size_t)S));
-    ROAM_TRY(ensure(c->assign_scratch, assign_scratch_bytes((uint32_t)S, (int64_t)c->g.bx * c->g.by * c->g.bz)));
-    launch_assign(c->cells.p, c->n_words, c->g.gx, c->g.gy, c->g.gz, (uint32_t)S, n_fields, c->assign_vox.p,
-                  labels, boxes, c->assign_scratch.p, c->n_sm, s);
+    ROAM_TRY(ensure(c->assign_scratch, assign_scratch_bytes((uint32_t)S, c->n_bricks)));
+    launch_assign(c->cells.p, c->n_words, c->g.gx, c->g.gy, c->g.gz, (uint32_t)S, c->n_bricks, n_fields,
+                  c->assign_vox.p, labels, boxes, c->assign_scratch.p, c->n_sm, s);
     ROAM_TRY(launched("field assignment"));
     ROAM_CUDA(cudaStreamSynchronize(s));
     if (assign_status(c->assign_scratch.p)) return fail(ROAM_ERR_DATA, "field assignment ran out of voxels");

@@ -59,3 +59,29 @@ def test_round_samples(tmp_path):
                            " (long long)round_samples(n, R, false));")
     for n, R, first, later in rows:
         assert first == n * min(R, 16) and later == first // 8
+
+
+# voxels, non-empty bricks, voxels per network, us per network from the lists and in the general form (GB300)
+ASSIGN = [
+    (190528, 2368, 17320, 27.0, 57.7), (190528, 2368, 95264, 71.3, 61.7),
+    (1524224, 18944, 3810, 14.5, 62.9), (1524224, 18944, 33135, 49.2, 74.5), (1524224, 18944, 138565, 133.3, 109.0),
+    (6193664, 86528, 15484, 34.4, 115.1), (6193664, 86528, 65196, 88.5, 133.1), (6193664, 86528, 269289, 274.2, 211.9),
+    (32768, 64, 2048, 12.1, 47.9), (262144, 512, 8192, 29.6, 52.5), (262144, 512, 131072, 76.7, 66.3),
+    (2097152, 4096, 33288, 52.9, 81.2), (2097152, 4096, 262144, 187.0, 136.6),
+    (16777216, 32768, 65027, 96.4, 244.9), (16777216, 32768, 1048576, 819.4, 529.5),
+    (41572, 4096, 8314, 20.2, 54.6), (32978, 20824, 2061, 23.0, 48.8), (32978, 20824, 16489, 101.5, 53.7),
+    (326729, 32764, 8168, 26.5, 53.3), (326729, 32764, 36303, 108.5, 68.1),
+    (267747, 168116, 2013, 35.3, 49.9), (267747, 168116, 16734, 117.8, 57.9), (267747, 168116, 66936, 376.0, 63.5),
+    (1985061, 262026, 8004, 48.9, 71.4), (1985061, 262026, 33084, 148.4, 85.6),
+    (99969, 83304, 2040, 30.8, 50.0), (99969, 83304, 16661, 132.7, 59.5),
+    (1998122, 1289647, 4995, 150.3, 83.9), (1998122, 1289647, 66604, 511.3, 120.5),
+    (19815086, 2097005, 65181, 389.3, 371.6), (19815086, 2097005, 1042899, 3431.2, 915.1),
+]
+
+
+def test_assignment_takes_the_form_measured_faster(tmp_path):
+    calls = "".join(f"show({S}, {B}, {per});" for S, B, per, _, _ in ASSIGN)
+    rows = _rows(tmp_path, "auto show = [](long long S, long long b, long long per) {"
+                           ' printf("%d\\n", (int)assign_from_bricks(S, b, per)); };' + calls)
+    for (S, B, per, lists, general), (chosen,) in zip(ASSIGN, rows):
+        assert (lists if chosen else general) <= 1.1 * min(lists, general), (S, B, per)

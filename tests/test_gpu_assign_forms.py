@@ -1,7 +1,9 @@
 """Both forms of the field assignment beyond the sizes of the other tests,
 against the oracle's full sort (labels equal, voxel for voxel; boxes equal):
 squared distances past 2^21, where the general form's key takes a fifth
-digit."""
+digit; and, from the brick lists, a first anchor so far from the rest that
+every brick is a candidate of its network: more than a block's table holds or
+just fewer, with a few voxels each or with many."""
 import numpy as np
 import pytest
 
@@ -54,4 +56,18 @@ def test_clusters_far_apart(roam, n):
     and 3: networks above 65,536 voxels; 40: small ones)."""
     dims = (2048, 2048, 8)
     lin = np.concatenate([_box(dims, (0, 0, 0), (90, 90, 8)), _box(dims, (1900, 1880, 0), (2040, 2030, 8))])
+    _check(roam, dims, lin, n)
+
+
+@pytest.mark.parametrize("x1,count,n", [
+    (2040, 60_000, 25),       # past the table, 2 voxels per brick
+    (2040, 300_000, 20),      # past the table, 9 voxels per brick
+    (1664, 45_000, 25),       # within the table, 4 voxels per brick, too many to keep in registers
+    (1664, 150_000, 20),      # within the table, 15 voxels per brick
+])
+def test_every_brick_a_candidate(roam, x1, count, n):
+    dims = (2048, 512, 64)
+    rng = np.random.default_rng(count)
+    x, y, z = rng.integers(1504, x1, count), rng.integers(0, 512, count), rng.integers(0, 64, count)
+    lin = np.concatenate([_box(dims, (0, 0, 0), (5, 4, 3)), (z * dims[1] + y) * dims[0] + x])
     _check(roam, dims, lin, n)
