@@ -41,7 +41,6 @@
 // All state stays on the device: no host synchronisation per network.
 #include <cooperative_groups.h>
 
-#include "dispatch.cuh"
 #include "internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -688,15 +687,16 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kAT, 1)
 
 }  // namespace
 
-// state and histogram, then (for the brick form) the lists
-size_t assign_scratch_bytes(uint32_t S, int64_t n_bricks)
+// state and histogram, then the lists
+size_t assign_scratch_bytes(uint32_t S, int64_t n_bricks, bool lists)
 {
-    const size_t nb = (size_t)n_bricks;
-    return sizeof(AssignState) + kBins * sizeof(uint32_t) + 16 + nb * 16 + 4 * kCluster + (size_t)S * 6;
+    return sizeof(AssignState) + kBins * sizeof(uint32_t) + 16 +
+           (lists ? (size_t)n_bricks * 16 + 4 * kCluster + (size_t)S * 6 : 0);
 }
 
 void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, uint32_t S, int64_t n_bricks,
-                   int n, uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm, cudaStream_t s)
+                   int n, bool lists, uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm,
+                   cudaStream_t s)
 {
     AssignState *st = reinterpret_cast<AssignState *>(scratch);
     uint32_t *hist = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(scratch) + sizeof(AssignState));
@@ -706,7 +706,7 @@ void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, 
     k_occupied_list<<<n_sm * 8, 256, 0, s>>>(cells, n_words, vox);
     const uint32_t per = S / (uint32_t)n;
     const int grid = n_sm * 4;
-    if (n > 1 && assign_from_bricks(S, n_bricks, per)) {
+    if (n > 1 && lists) {
         const size_t nb = (size_t)n_bricks;
         BrickLists L;
         L.n = hist + kBins;

@@ -274,10 +274,11 @@ void launch_teacher_simt(const float *wt, TeacherAffine aff, int64_t n, const fl
                          int n_sm, cudaStream_t s);
 void launch_distill_loss(int64_t n, const float4 *student, const float4 *teacher, float I, float4 *dl, float *loss,
                          cudaStream_t s);
-size_t assign_scratch_bytes(uint32_t S, int64_t n_bricks);
-// n_bricks: 8^3 bricks with an occupied voxel
+// n_bricks: 8^3 bricks with an occupied voxel; lists: from brick lists (they need their scratch)
+size_t assign_scratch_bytes(uint32_t S, int64_t n_bricks, bool lists);
 void launch_assign(const uint2 *cells, int64_t n_words, int gx, int gy, int gz, uint32_t S, int64_t n_bricks,
-                   int n, uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm, cudaStream_t s);
+                   int n, bool lists, uint32_t *vox, uint16_t *field, int32_t *boxes, void *scratch, int n_sm,
+                   cudaStream_t s);
 uint32_t assign_status(const void *scratch);
 size_t occupancy_view_bytes(int n_views);
 // per view: what its rays share (`views`), and the sines and cosines of its

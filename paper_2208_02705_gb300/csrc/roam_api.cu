@@ -1258,8 +1258,11 @@ roam_status roam_assign_fields(roam_ctx *c, int n_fields, uint16_t *labels, int3
     if (S >= (int64_t)1 << 27) return fail(ROAM_ERR_ARG, "at most 2^27 - 1 occupied voxels");
     cudaStream_t s = (cudaStream_t)stream;
     ROAM_TRY(ensure(c->assign_vox, (size_t)S));
-    ROAM_TRY(ensure(c->assign_scratch, assign_scratch_bytes((uint32_t)S, c->n_bricks)));
-    launch_assign(c->cells.p, c->n_words, c->g.gx, c->g.gy, c->g.gz, (uint32_t)S, c->n_bricks, n_fields,
+    // (without memory for the lists the general form serves)
+    bool lists = n_fields > 1 && assign_from_bricks(S, c->n_bricks, S / n_fields);
+    if (lists) lists = ensure(c->assign_scratch, assign_scratch_bytes((uint32_t)S, c->n_bricks, true)) == ROAM_OK;
+    if (!lists) ROAM_TRY(ensure(c->assign_scratch, assign_scratch_bytes((uint32_t)S, c->n_bricks, false)));
+    launch_assign(c->cells.p, c->n_words, c->g.gx, c->g.gy, c->g.gz, (uint32_t)S, c->n_bricks, n_fields, lists,
                   c->assign_vox.p, labels, boxes, c->assign_scratch.p, c->n_sm, s);
     ROAM_TRY(launched("field assignment"));
     ROAM_CUDA(cudaStreamSynchronize(s));

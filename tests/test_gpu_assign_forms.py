@@ -71,3 +71,26 @@ def test_every_brick_a_candidate(roam, x1, count, n):
     x, y, z = rng.integers(1504, x1, count), rng.integers(0, 512, count), rng.integers(0, 64, count)
     lin = np.concatenate([_box(dims, (0, 0, 0), (5, 4, 3)), (z * dims[1] + y) * dims[0] + x])
     _check(roam, dims, lin, n)
+
+
+def test_lists_take_memory_only_where_they_are_used(roam):
+    """The general form (here: one network, and two of 4.2 M voxels) holds the
+    voxels' indices and a few kilobytes; the lists take 6 bytes per voxel more."""
+    dims = (256, 256, 128)
+    S = dims[0] * dims[1] * dims[2]
+    r = roam.Roam(0)
+    r.load_grid(np.full(S // 32, 0xffffffff, np.uint32), dims, (0.0, 0.0, 0.0), 0.1)
+    del_me = torch.empty(S, dtype=torch.int16, device="cuda")      # (the labels come from torch's cache below)
+    del del_me
+    torch.empty((600, 6), dtype=torch.int32, device="cuda")
+
+    def held(n):
+        free = torch.cuda.mem_get_info()[0]
+        r.assign_fields(n)
+        torch.cuda.synchronize()
+        return free - torch.cuda.mem_get_info()[0]
+
+    assert held(1) <= 4 * S + (8 << 20)
+    assert held(2) <= 8 << 20
+    assert held(600) >= 6 * S - (8 << 20)
+    r.close()
