@@ -69,7 +69,10 @@ __device__ __forceinline__ void st_words32(uint32_t tArow, int c, const uint32_t
 // slots' chains overlap.  Tiles come in field-uniform groups of kSlots (bucket padding);
 // at a field change all slots meet at a CTA barrier, thread 0 reloads the
 // shared weight image, and each issuer waits for it before its next MMA.
-template <int W, int H, bool F8, int kSlots, int CG>
+// kAnyPos: a position may be NaN or infinite.  Its encoding then is NaN, which
+// max(v, 0) ends in the first layer and the ReLU fused into the E4M3 conversion
+// does not (a render's positions are finite).
+template <int W, int H, bool F8, int kSlots, int CG, bool kAnyPos>
 __global__ void __launch_bounds__(kSlots * CG * 128, 1)
     k_mlp_tc(const void *wimg, int64_t img_bytes, int field_base, int cls, const float *affine, float sig_scale,
              int act, SampleSrc src, BucketBufs b, Counters *ctr, float4 *out, unsigned long long wait_ns,
@@ -312,6 +315,12 @@ __global__ void __launch_bounds__(kSlots * CG * 128, 1)
                             }
                         }
                     }
+                    if constexpr (kAnyPos) {
+                        if (l == 0) {
+#pragma unroll
+                            for (int q = 0; q < 32; ++q) v[q] = fmaxf(v[q], 0.f);
+                        }
+                    }
                     if (l == H) st_act32<F8, false>(tArow, c, v);
                     else st_act32<F8, true>(tArow, c, v);
                 }
@@ -515,17 +524,25 @@ __global__ void k_adam_tc(float *__restrict__ w, float *__restrict__ m, float *_
 template <int W, int H, bool F8>
 int tc_smem_bytes() { return 1024 + TcShape<W, H, F8>::kImageAlloc; }
 
-template <int W, int H, bool F8, int kSlots, int CG>
-void launch_form(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out, int n_sm,
+template <int W, int H, bool F8, int kSlots, int CG, bool kAnyPos>
+void launch_kernel(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out, int n_sm,
                cudaStream_t s)
 {
     const int smem = tc_smem_bytes<W, H, F8>();
     static int smem_set[kMaxDevices] = {};
-    raise_smem_limit((const void *)k_mlp_tc<W, H, F8, kSlots, CG>, smem, smem_set);
+    raise_smem_limit((const void *)k_mlp_tc<W, H, F8, kSlots, CG, kAnyPos>, smem, smem_set);
     const void *img = F8 ? w.wimg8 : w.wimg;
     const int64_t ib = F8 ? w.img8_bytes : w.img_bytes;
-    launch_pdl(k_mlp_tc<W, H, F8, kSlots, CG>, n_sm, kSlots * CG * 128, smem, s, img, ib, w.field_base, w.cls, w.affine,
+    launch_pdl(k_mlp_tc<W, H, F8, kSlots, CG, kAnyPos>, n_sm, kSlots * CG * 128, smem, s, img, ib, w.field_base, w.cls, w.affine,
                w.sigma_scale, w.act, src, b, ctr, out, w.wait_ns ? w.wait_ns : kWaitNs, w.withhold_image);
+}
+
+template <int W, int H, bool F8, int kSlots, int CG>
+void launch_form(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out, int n_sm,
+                 cudaStream_t s)
+{
+    if (F8 && src.mode != 0) launch_kernel<W, H, F8, kSlots, CG, F8>(w, src, b, ctr, out, n_sm, s);
+    else launch_kernel<W, H, F8, kSlots, CG, false>(w, src, b, ctr, out, n_sm, s);
 }
 
 // Tiles in flight (w.slots: as the tiles were padded) and warpgroups per slot.

@@ -256,8 +256,7 @@ __device__ __forceinline__ uint32_t pack_e4m3x4(float a, float b, float c, float
     return (uint32_t)lo | ((uint32_t)hi << 16);
 }
 
-// the same through a ReLU fused into the conversion (the inputs are never NaN:
-// s D + b with finite terms)
+// the same through a ReLU fused into the conversion (a NaN stays one)
 __device__ __forceinline__ uint32_t pack_e4m3x4_relu(float a, float b, float c, float d)
 {
     uint16_t lo, hi;
