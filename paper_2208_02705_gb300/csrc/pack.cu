@@ -127,13 +127,14 @@ __device__ __forceinline__ void pack_layer(const float *__restrict__ src, int l,
         }
         if (d.img8) {
             uint8_t *o = d.img8 + f * d.img8_bytes;
-            // channel scales: max |row| / 448 (1 for an all-zero row), a warp per row
+            // channel scales: max |row| / 448 (1 for an all-zero row; at least the
+            // smallest float, so that no weight becomes 0 / 0), a warp per row
             for (int r = tid >> 5; r < N; r += kPackThreads / 32) {
                 float m = 0.f;
                 for (int k = tid & 31; k < K; k += 32) m = fmaxf(m, fabsf(sm[r * LD + k]));
 #pragma unroll
                 for (int s = 16; s > 0; s >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, s));
-                if ((tid & 31) == 0) scale[r] = m > 0.f ? m / 448.0f : 1.f;
+                if ((tid & 31) == 0) scale[r] = m > 0.f ? fmaxf(m / 448.0f, __int_as_float(1)) : 1.f;
             }
             __syncthreads();
             for (int q = tid; q < S8::chunks(KIND == kHidden ? 1 : (KIND == kL1 ? 0 : (KIND == kHead ? H : H + 1))) * NM * 8;

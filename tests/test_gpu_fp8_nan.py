@@ -59,3 +59,27 @@ def test_positions_without_a_finite_encoding(roam, W, H):
     assert torch.isfinite(out).all()
     r.close()
     r0.close()
+
+
+@pytest.mark.parametrize("W,H", [(32, 2), (64, 2), (128, 2)])
+def test_rows_whose_scale_underflows(roam, W, H):
+    """An output whose weights are zeros and values below 448 times the smallest
+    float: its scale max / 448 would round to 0 and 0 / 0 make its weights NaN.
+    Such weights add nothing to a bias that is not as small, so the outputs are
+    those of a row of zeros, bit for bit."""
+    w = F.xavier_weights(2, F.ROLE_STUDENT, FIELDS, W, H, bias_scale=0.3)
+    hidden = W * 63 + W                       # H = 2: one hidden layer, [out][in]
+    w0 = w.copy()
+    for row in (0, W // 2, W - 1):
+        s = slice(hidden + row * W, hidden + (row + 1) * W)
+        w0[:, s] = 0.0
+        w[:, s] = 0.0
+        w[:, hidden + row * W + 3] = np.float32(1e-43)
+        w[:, hidden + row * W + 5] = np.float32(-2.8e-45)
+    p, d, f = _points(300, W)
+    r, r0 = _ctx(roam, w, W, H), _ctx(roam, w0, W, H)
+    out, ref = r.mlp_eval(p, d, f, roam.ROAM_FP8), r0.mlp_eval(p, d, f, roam.ROAM_FP8)
+    assert torch.isfinite(ref).all()
+    assert torch.equal(out, ref)
+    r.close()
+    r0.close()
