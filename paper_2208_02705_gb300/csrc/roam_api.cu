@@ -1,5 +1,7 @@
 // C ABI of the roam library: argument validation, device memory of the
 // context, and the order of kernel launches for each entry point.
+#include <cuda.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
@@ -721,6 +723,33 @@ roam_status set_field_order(roam_ctx *c, const uint16_t *perm)
     return ROAM_OK;
 }
 
+// Whether [p, p + bytes) lies within one allocation of this device's memory, so
+// that a kernel may read it.
+bool in_device_memory(const void *p, size_t bytes, int device)
+{
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (at.type != cudaMemoryTypeDevice || at.device != device) return false;
+    using Range = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const Range range = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found{};
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<Range>(fn);
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    return range && range(&base, &size, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS &&
+           (uintptr_t)p - (uintptr_t)base + bytes <= size;
+}
+
 // Loads weight set k: n fields of width W (internal ids first .. first + n - 1),
 // FP32 masters in the API layout, and packs the SIMT and tensor-core copies.
 roam_status load_set(roam_ctx *c, int k, int W, int H, int first, int n, const float *weights, bool on_device)
@@ -744,11 +773,15 @@ roam_status load_set(roam_ctx *c, int k, int W, int H, int first, int n, const f
     ROAM_TRY(ensure(q.wr, (size_t)(q.Pr * n)));
     if (q.tc_ok) ROAM_TRY(ensure(q.wimg, (size_t)(q.img_bytes * n)));
     if (q.tc8_ok) ROAM_TRY(ensure(q.wimg8, (size_t)(q.img8_bytes * n)));
-    // device weights are read once, by the pass that writes the masters and
-    // every copy of them
-    if (!on_device) ROAM_CUDA(cudaMemcpy(q.w32.p, weights, total * sizeof(float), cudaMemcpyHostToDevice));
+    // weights in this device's memory are read once, by the pass that writes the
+    // masters and every copy of them; any others go through a copy, which also
+    // refuses what it cannot read
+    const bool direct = on_device && in_device_memory(weights, (size_t)total * sizeof(float), c->device);
+    if (!direct)
+        ROAM_CUDA(cudaMemcpy(q.w32.p, weights, total * sizeof(float),
+                             on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice));
     PackDst d{};
-    d.w32 = on_device ? q.w32.p : nullptr;
+    d.w32 = direct ? q.w32.p : nullptr;
     d.wt = q.wt.p;
     d.wr = q.wr.p;
     d.img = q.tc_ok ? q.wimg.p : nullptr;
@@ -757,7 +790,7 @@ roam_status load_set(roam_ctx *c, int k, int W, int H, int first, int n, const f
     d.img8_bytes = q.img8_bytes;
     d.bad = c->d_flag;
     ROAM_CUDA(cudaMemset(c->d_flag, 0, 4));
-    launch_pack(on_device ? weights : q.w32.p, n, W, H, P, d, 0);
+    launch_pack(direct ? weights : q.w32.p, n, W, H, P, d, 0);
     ROAM_TRY(launched("weight pack"));
     uint32_t bad = 0;
     ROAM_CUDA(cudaMemcpy(&bad, c->d_flag, 4, cudaMemcpyDeviceToHost));
