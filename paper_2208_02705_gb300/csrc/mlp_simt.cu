@@ -1,11 +1,11 @@
 // FP32 SIMT evaluation of the per-field tiny MLPs (the plain FP32 form of
-// querying many MLPs at once): a block of 8 warps takes one tile of 128
-// samples of one field at a time, each layer a register-tiled FP32 product.
+// querying many MLPs at once): a block of 8 warps (4 at W = 32) takes one tile of
+// 128 samples of one field at a time, each layer a register-tiled FP32 product.
 //
 // What bounds it: the FP32 FMA pipe, and beside it the register writes of the
 // shared-memory loads (a float4 read from shared memory costs the FMA pipe of
 // its sub-partition about 5 cycles).  So a thread owns TS samples x TN outputs
-// (4 x 4 at W = 32, 4 x 8 at W = 64, 8 x 8 at W = 128) as packed FMAs; the
+// (8 x 4 at W = 32, 4 x 8 at W = 64, 8 x 8 at W = 128) as packed FMAs; the
 // layer's input sits in shared memory feature-major (rows of 128 samples,
 // padded by 4), and its outputs replace it in place.  The weights (transposed
 // copy, [in][out]) stream through a ring of 16-row stages copied asynchronously
@@ -13,25 +13,31 @@
 // weights beside it, and two or three blocks share an SM: while one waits at
 // a barrier or encodes, the others multiply.  Measured (GB300), against the
 // field's weights beside two tiles of 4 warps in one block per SM: 8.2 M samples
-// at W = 64 / H = 3 8.81 -> 7.90 ms (0.58 of the FP32 peak), 2.1 M at W = 32 / H = 2
-// 1.04 -> 0.79 ms, 2.1 M at W = 128 / H = 3 8.56 -> 6.04 ms; 79,000 samples over
-// 512 fields 213 -> 116 us.
+// of a render at W = 64 / H = 3 8.83 -> 7.86 ms (0.58 of the FP32 peak), 8.4 M at
+// W = 32 / H = 2 3.29 -> 2.86 ms, 8.2 M at W = 128 / H = 3 28.6 -> 23.2 ms; 5,000
+// points of 1024 fields at W = 64 / H = 3 235 -> 109 us.  Where fields have long
+// runs, so that the replaced form rarely reloaded its weights, the two are level:
+// 32.7 M samples of 64 fields at W = 32 / H = 4 13.73 and 13.74 ms, 1 M points of
+// one field there 430 and 446 us.
 #include "simt_common.cuh"
 
 namespace roam {
 
 namespace {
 
-constexpr int kThreads = 256;
 constexpr int kTile = 128;            // samples per tile
 constexpr int XS = kTile + 4;         // row stride of the activations
 constexpr int kRingRows = 16, kStages = 3;
 
 template <int W, int H>
 struct SimtShape {
-    static constexpr int TS = W == 128 ? 8 : 4;                  // samples per thread
+    static constexpr int kThreads = W == 32 ? 128 : 256;
+    static constexpr int TS = W == 64 ? 4 : 8;                   // samples per thread
     static constexpr int TN = kTile * W / (kThreads * TS);       // outputs per thread
     static constexpr int SB = kTile / (8 * TS);                  // warps along the samples
+    // warps without samples in a part-filled tile skip its products (at W = 128
+    // the test spills more accumulators: 2 % of full tiles)
+    static constexpr bool kSkip = W < 128;
     static constexpr int NH = round4(1 + W);
     static constexpr int rX = W >= 64 ? 0 : round4(W + kPeD);    // rows of F(x): beside those of [h; F(d)] at W = 32
     static constexpr int kRows = W >= 64 ? W + kPeD : rX + kPeX;
@@ -40,9 +46,9 @@ struct SimtShape {
     static constexpr int kPer = (kPeX + kRingRows - 1) / kRingRows + H * ((W + kRingRows - 1) / kRingRows) +
                                 (W + kPeD + kRingRows - 1) / kRingRows + 1;
     static constexpr size_t kSmem = (size_t)(kRows * XS + kStages * kStage + 4 * kTile) * sizeof(float);
-    // per SM: what registers hold without spilling the accumulators (at W = 64 a
-    // third block at 80 registers measured 0.5 % faster on a full chip and 7 %
-    // slower on few tiles)
+    // per SM: what shared memory holds (W = 32), or registers without spilling
+    // the accumulators (at W = 64 a third block at 80 registers measured 0.5 %
+    // faster on a full chip and 7 % slower on few tiles)
     static constexpr int kBlocks = W == 32 ? 3 : 2;
     static_assert(kRows >= kPeX && TN % 4 == 0, "whole float4 runs per thread");
 };
@@ -51,11 +57,12 @@ __device__ __forceinline__ float softplus_f(float s) { return s > 20.f ? s : log
 __device__ __forceinline__ float sigmoid_f(float s) { return 1.f / (1.f + expf(-s)); }
 
 template <int W, int H>
-__global__ void __launch_bounds__(kThreads, SimtShape<W, H>::kBlocks)
+__global__ void __launch_bounds__(SimtShape<W, H>::kThreads, SimtShape<W, H>::kBlocks)
     k_mlp_simt(MlpWeights w, SampleSrc src, BucketBufs b, Counters *ctr, float4 *out)
 {
     using F = SimtShape<W, H>;
-    constexpr int TS = F::TS, TN = F::TN, G = TS / 4, KC = W + kPeD;
+    constexpr int TS = F::TS, TN = F::TN, G = TS / 4, KC = W + kPeD, kThreads = F::kThreads;
+    constexpr int NP = kThreads / kTile;               // threads per sample in the gather and the output layer
     constexpr TLayout TL(W, H);
     extern __shared__ float4 smem4[];
     __shared__ int2 entries[F::kPer];                  // a tile's ring stages: offset in wt, 16-byte pieces
@@ -126,6 +133,7 @@ __global__ void __launch_bounds__(kThreads, SimtShape<W, H>::kBlocks)
     const int s0 = (warp % F::SB) * 8 * TS + 4 * sg;
     const int n0 = (warp / F::SB) * 4 * TN + og * TN;
     const bool dens_warp = warp / F::SB == 0;           // the warps that also form the density logit
+    bool live = true;                                   // the warp's samples reach into the tile
 
     // rows [0, K) x [K][LD] weights -> acc; kDens: also dens from column W
     auto dense = [&](auto KK, auto LDc, auto DENS, const float *x, float2 (&acc)[SimtShape<W, H>::TS][SimtShape<W, H>::TN / 2], float (&dens)[SimtShape<W, H>::TS]) {
@@ -156,12 +164,17 @@ __global__ void __launch_bounds__(kThreads, SimtShape<W, H>::kBlocks)
                 }
             }
         };
+        if (F::kSkip && !live) {                        // (the stages' barriers are everyone's)
+#pragma unroll 1
+            for (int k0 = 0; k0 < K; k0 += kRingRows) next_stage();
+            return;
+        }
 #pragma unroll 1
         for (int k0 = 0; k0 + kRingRows <= K; k0 += kRingRows) rows(Int<kRingRows>{}, k0);
         if constexpr (K % kRingRows != 0) rows(Int<K % kRingRows>{}, K - K % kRingRows);
     };
 
-    const int smp = tid & 127, part = tid >> 7;          // two threads per sample in the gather and the output layer
+    const int smp = tid & (kTile - 1), part = tid / kTile;
     SimtPending pend{};
     simt_index(pend, b, tl, smp, true);
     simt_record(pend, src);
@@ -184,7 +197,9 @@ __global__ void __launch_bounds__(kThreads, SimtShape<W, H>::kBlocks)
         };
         load_bias(TL.l1 + kPeX * W);
         const float bd = __ldg(wf + TL.head + W * F::NH + W);
-        simt_encode<2, XS>(me, src, w.affine + 6 * (int64_t)tc.field, X + F::rX * XS + smp, X + W * XS + smp, part);
+        live = (uint32_t)((warp % F::SB) * 8 * TS) < tc.count;
+        if (!F::kSkip || (uint32_t)(smp & ~31) < tc.count)
+            simt_encode<NP, XS>(me, src, w.affine + 6 * (int64_t)tc.field, X + F::rX * XS + smp, X + W * XS + smp, part);
         float dens[TS];
         // one layer in place: rows [0, W) become its outputs (the first stage's
         // barrier orders them after what wrote the input)
@@ -230,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, SimtShape<W, H>::kBlocks)
         }
         layer(Int<KC>{}, Int<W>{}, Int<0>{}, X, true, -1);
         simt_ray(pend, src);
-        // ---- rgb = sigmoid(Wo g + bo): a sample's two threads take half of the sums each ----
+        // ---- rgb = sigmoid(Wo g + bo): a sample's threads take their shares of the sums ----
         {
             const float4 *wo = reinterpret_cast<const float4 *>(next_stage());     // [W][4], then bias[4]
             float z[3] = {0.f, 0.f, 0.f};
@@ -240,16 +255,16 @@ __global__ void __launch_bounds__(kThreads, SimtShape<W, H>::kBlocks)
                 z[1] = bo.y;
                 z[2] = bo.z;
             }
-            const float *g = X + part * (W / 2) * XS + smp;
+            const float *g = X + part * (W / NP) * XS + smp;
 #pragma unroll 8
-            for (int k = 0; k < W / 2; ++k) {
-                const float4 wk = wo[part * (W / 2) + k];
+            for (int k = 0; k < W / NP; ++k) {
+                const float4 wk = wo[part * (W / NP) + k];
                 const float gk = g[k * XS];
                 z[0] = fmaf(wk.x, gk, z[0]);
                 z[1] = fmaf(wk.y, gk, z[1]);
                 z[2] = fmaf(wk.z, gk, z[2]);
             }
-            if (part == 1) {
+            if (NP > 1 && part == 1) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) red[c * kTile + smp] = z[c];
             }
@@ -257,8 +272,11 @@ __global__ void __launch_bounds__(kThreads, SimtShape<W, H>::kBlocks)
             if (part == 0 && me.on) {
                 const float sl = red[3 * kTile + smp];
                 const float sigma = w.sigma_scale * (w.act == ROAM_RELU ? fmaxf(sl, 0.f) : softplus_f(sl));
-                out[me.idx] = make_float4(sigma, sigmoid_f(z[0] + red[smp]), sigmoid_f(z[1] + red[kTile + smp]),
-                                          sigmoid_f(z[2] + red[2 * kTile + smp]));
+                if constexpr (NP > 1) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) z[c] += red[c * kTile + smp];
+                }
+                out[me.idx] = make_float4(sigma, sigmoid_f(z[0]), sigmoid_f(z[1]), sigmoid_f(z[2]));
             }
         }
     }
@@ -274,7 +292,7 @@ static void launch_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs
     static int smem_set[kMaxDevices] = {};
     raise_smem_limit((const void *)k_mlp_simt<W, H>, (int)F::kSmem, smem_set);
     // one wave of resident blocks; each takes a contiguous run of tiles
-    launch_pdl(k_mlp_simt<W, H>, n_sm * F::kBlocks, kThreads, F::kSmem, s, w, src, b, ctr, out);
+    launch_pdl(k_mlp_simt<W, H>, n_sm * F::kBlocks, F::kThreads, F::kSmem, s, w, src, b, ctr, out);
 }
 
 void launch_mlp_simt(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out,

@@ -107,7 +107,8 @@ __device__ __forceinline__ void simt_encode(const SimtPending &me, const SampleS
     if (part == 0) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) xp[a * XS] = xl[a];
-    } else if (part == 1) {
+    }
+    if (part == (NP > 1 ? 1 : 0)) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) dp[a * XS] = dv[a];
     }
