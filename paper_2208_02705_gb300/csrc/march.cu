@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(256) k_march(GridDev g, MarchParams p)
         const uint32_t R = (uint32_t)p.R, n_max = (uint32_t)p.n_max;
         // records this round may keep (the round's size and the ray's budget in one bound)
         const uint32_t lim = nk < n_max ? min(R, n_max - nk) : 0u;
-        // slot of record em: s0 + em * s_step
+        // the next record's slot, and from one to the next
         uint32_t at = p.flat ? i * R : slot_of(i, 0u, R);
         const uint32_t s_step = p.flat ? 1u : 32u;
         // the histogram takes runs of one field (a ray crosses few fields),

@@ -546,14 +546,14 @@ void launch_form(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b,
 }
 
 // Tiles in flight (w.slots: as the tiles were padded) and warpgroups per slot.
-// TMEM admits only two slots at W = 128, whose epilogues
-// leave most issue slots empty with one warpgroup each; but two, at 128
-// registers a thread where one takes 152, hide less of a gather's latency.  FP8:
-// two (8.2 M samples of a render at H = 3 2009 -> 1952 us, 4 M scattered points
-// 1114 -> 1070).  BF16: two for rays, whose samples lie together in memory
-// (the same render 1940 -> 1852 us), one for direct points, which a caller may
-// have in any order (4 M scattered points of 128 fields at H = 4: 1135 us, 1245
-// with two; points in field order 1200 and 1117).
+// TMEM admits only two slots at W = 128, whose epilogues leave most issue slots
+// empty with one warpgroup each; but two, at 128 registers a thread where one
+// takes 152, hide less of a gather's latency.  FP8: two (8.2 M samples of a render
+// at H = 3 2009 -> 1952 us, 4 M scattered points 1114 -> 1070).  BF16: two for
+// rays, whose samples lie together in memory (the same render 1940 -> 1852 us),
+// one for direct points, which a caller may have in any order (4 M scattered
+// points of 128 fields at H = 4: 1133 us, 1245 with two; points in field order
+// 1200 and 1117).
 template <int W, int H, bool F8>
 void launch_t(const MlpWeights &w, const SampleSrc &src, const BucketBufs &b, Counters *ctr, float4 *out, int n_sm,
               cudaStream_t s)

@@ -301,7 +301,7 @@ bool all_tc(const roam_ctx *c, bool f8)
 
 // Derived weight copies that an Adam step left stale are rebuilt before the
 // first launch that reads them: the SIMT forward's transposed copy (FP32
-// forward or SIMT adjoint), the SIMT adjoint's row-padded copy, the FP8
+// forward or SIMT adjoint), the SIMT adjoint's dgrad copy, the FP8
 // images.  Adam rebuilds the BF16 images itself.
 constexpr uint32_t kStaleWt = 1u, kStaleWr = 2u, kStaleImg8 = 4u;
 
